@@ -242,8 +242,9 @@ qf_status qf_sweep_run_items(const qf_state* st, uint64_t* items, size_t cap, si
  * framework's caching pool, a serving process with a fixed memory budget), or
  * in a latency-critical loop that must not take cudaMalloc's implicit device
  * synchronisation.  qf_expectation needs a qf_state, whose creation allocates;
- * this call computes the same <psi|H|psi> (same kernel, same precision) from
- * amplitudes the caller owns.
+ * this call computes the same <psi|H|psi> (same precision; equal within rounding:
+ * from 15 qubits on qf_expectation may sum in another order) from amplitudes the
+ * caller owns.
  *   amplitudes: device pointer to 2^n amplitudes in the layout above (the state
  *     itself, no separate scale), 16-byte aligned; not modified.
  *   stream: cudaStream_t the work is queued on (NULL = legacy default stream);

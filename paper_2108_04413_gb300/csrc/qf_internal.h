@@ -89,6 +89,37 @@ struct __align__(256) RealChunk {
   float tf[1 << kChunkTerms];  // the same weights in FP32 (complex64 states)
 };
 
+// Expectation passes: a pass is a set S of tile bits (2^s amplitudes per tile) and
+// the X-mask groups whose x lies in S, so that a tile staged in shared memory once
+// serves all of them.  Each group's masks are kept in tile-local bit positions.
+constexpr int kPassThreads = 256;
+constexpr int kPassGroups = 128;  // groups of one pass (their records sit in shared memory)
+constexpr int kPassMaxChunk = 1 << 12;  // a group of this many chunks takes the per-group kernel
+// Per real type: tile bits S, low contiguous bits L (128 bytes), a thread's pairs P
+// and how many of them are summed before they join the thread's total.
+template <typename T> struct PassTile;
+template <> struct PassTile<double> { static constexpr int S = 12, L = 3, P = 1 << (S - 9), B = P; };
+template <> struct PassTile<float> { static constexpr int S = 13, L = 4, P = 1 << (S - 9), B = 4; };
+struct ExpPass {
+  int g0, g1;         // PassGroups [g0, g1)
+  uint8_t sbits[16];  // the tile's bit positions, ascending
+};
+struct PassGroup {
+  uint32_t xl;        // x in tile-local bits
+  int hl;             // highest set bit of xl, -1 for the diagonal group
+  int chunk;          // first PassChunk; also the first ExpChunk of the group's tables
+  int nchunk_flags;   // nchunk << 3 | ExpGroup::flags
+};
+// One chunk's masks split into tile-local bits and the rest.  A thread visits the
+// tile-local indices j0 + o_k (no common bits; o_k the same for every thread), so a
+// term's sign is the parity of (its mask & j0), of (its outside mask & the tile) and
+// of (its mask & o_k); the last is bit t of nibble k of kx.
+struct PassChunk {
+  uint64_t zout[kChunkTerms];
+  uint32_t zl[kChunkTerms];
+  uint64_t kx[2];     // nibbles k = 0..15, 16..31
+};
+
 // H|psi> plan (tiled): groups sorted by X mask form classes of equal high part
 // x >> tb (tb = tile bits); a class reads one partner tile per output tile.
 constexpr int kWideTerms = 8;  // terms per H|psi> sign-pattern table
@@ -307,6 +338,12 @@ bool sparse_q_imag(const SparseArgs& a);
 cudaError_t launch_expect(const void* psi, int n, qf_dtype dt, const ExpGroup* groups, int ngroups,
                           const ExpChunk* chunks, double* partials, unsigned* counter, double* out,
                           int nblocks, cudaStream_t s);
+// The same for groups gathered into passes (n >= PassTile::S): tabs are the plan's
+// ExpChunks.  Weak: a build of the planner without the kernels takes launch_expect.
+__attribute__((weak)) cudaError_t launch_expect_passes(const void* psi, int n, qf_dtype dt, const ExpPass* passes,
+                                                       int npass, const PassGroup* groups, const PassChunk* chunks,
+                                                       const ExpChunk* tabs, double* partials, int max_blocks,
+                                                       unsigned* counter, double* out, cudaStream_t s);
 // lam = H psi, out[0] = Re <psi|lam>, out[1] = <psi|psi>; partials holds 2 * nblocks doubles.
 cudaError_t launch_hpsi(const void* psi, void* lam, int n, qf_dtype dt, const ExpGroup* groups, int ngroups,
                         const ExpChunk* chunks, double* partials, unsigned* counter, double* out, int nblocks,

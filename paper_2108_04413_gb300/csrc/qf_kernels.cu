@@ -12,6 +12,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "qf_internal.h"
@@ -616,6 +617,250 @@ __global__ void __launch_bounds__(256) k_expect_tiled(const typename Cx<T>::V* _
     }
   }
   grid_finish(acc, partials, counter, out);
+}
+
+// Passes (ExpPass): a CTA stages a tile of 2^S amplitudes (64 KB) in shared memory
+// with asynchronous copies and evaluates every group of the pass on it, so the
+// state is read once per pass instead of once per group (28 qubits, 500 strings: 53
+// reads instead of 440); three CTAs per SM overlap one's copies with the others'
+// sums.
+// complex128 is bound by the FP64 pipe: two multiply-adds per pair and group, 75.6 ms
+// of the 91.5 ms that 25 qubits, 1500 terms take (236 ms in the per-group kernel).
+// complex64 is bound by shared-memory bandwidth (16 bytes per pair and group, 23 ms
+// of the 46 ms that 28 qubits, 500 terms take; 178 ms in the per-group kernel) and,
+// in passes of few groups, by the state's reads (53 reads: 17 ms); taking such passes
+// in turn with large ones tile by tile was slower (56 ms: spills).
+// complex64 sums stay in FP32 over four pairs, then join a float pair by TwoSum
+// (converted to FP64 once per tile).
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() {
+  asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+}
+
+template <typename T> struct PassAcc {  // FP64 state: one running sum
+  double s = 0.0;
+  __device__ __forceinline__ void add(double w, double v) { s = fma(w, v, s); }
+  __device__ __forceinline__ void add(double v) { s += v; }
+  __device__ __forceinline__ double take() {
+    const double v = s;
+    s = 0.0;
+    return v;
+  }
+};
+template <> struct PassAcc<float> {
+  float h = 0.f, l = 0.f;
+  __device__ __forceinline__ void add(float w, float v) { add(w * v); }
+  __device__ __forceinline__ void add(float v) {  // TwoSum, the error into l
+    const float t = __fadd_rn(h, v);
+    const float bp = __fsub_rn(t, h);
+    l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(t, bp)), __fsub_rn(v, bp)));
+    h = t;
+  }
+  __device__ __forceinline__ double take() {
+    const double v = (double)h + (double)l;
+    h = l = 0.f;
+    return v;
+  }
+};
+
+template <typename T> __device__ __forceinline__ T pass_weight(const ExpChunk* C, unsigned i, bool im);
+template <> __device__ __forceinline__ double pass_weight<double>(const ExpChunk* C, unsigned i, bool im) {
+  return im ? __ldg(&C->tab[i].y) : __ldg(&C->tab[i].x);
+}
+template <> __device__ __forceinline__ float pass_weight<float>(const ExpChunk* C, unsigned i, bool im) {
+  return im ? __ldg(&C->ftab[i].y) : __ldg(&C->ftab[i].x);
+}
+
+// A thread's pairs of a group with pivot bit hl: j = j0 + o_k and j ^ xl, o_k running
+// over the tile bits above the thread's own.  Those bits depend only on the case
+// C = max(0, hl - 8) (the thread's 8 bits spread over bits 0..8 around a pivot up to
+// bit 8, else the high bits leave out the pivot), so o_k is a constant: one load
+// with an immediate offset and one XOR for the partner's address.
+template <typename T, int C> struct PassPairs {
+  static constexpr int P = PassTile<T>::P, KB = PassTile<T>::S - 9;
+  static __device__ __forceinline__ unsigned off(int k) {
+    unsigned o = 0;
+#pragma unroll
+    for (int i = 0; i < KB; ++i)
+      if ((k >> i) & 1) o |= 1u << (C == 0 ? 9 + i : 8 + i < 8 + C ? 8 + i : 9 + i);
+    return o;
+  }
+  template <typename F>
+  static __device__ __forceinline__ void run(const unsigned char* tile, unsigned j0, unsigned xl, F&& f) {
+    using V = typename Cx<T>::V;
+    const unsigned a = j0 * sizeof(V), b = (j0 ^ xl) * sizeof(V);
+#pragma unroll
+    for (int k = 0; k < P; ++k) {
+      const unsigned o = off(k) * (unsigned)sizeof(V);
+      f(k, *reinterpret_cast<const V*>(tile + a + o), *reinterpret_cast<const V*>(tile + (b ^ o)));
+    }
+  }
+};
+
+// One-term group: the sum over the thread's pairs of +-Re w (+-Im w) times the term's
+// weight w, which carries the thread's own sign.  Nibble 2^i of km is the sign of
+// bit i of k; the sign of pair k is their product.
+template <typename T, int C, bool IM>
+__device__ __forceinline__ void pass_single(const unsigned char* tile, unsigned j0, unsigned xl, uint64_t km, T w,
+                                            PassAcc<T>& acc) {
+  using V = typename Cx<T>::V;
+  if constexpr (sizeof(T) == 8) {  // two multiply-adds per pair, the sign on the amplitude
+    T g = T(0);
+    PassPairs<T, C>::run(tile, j0, xl, [&](int k, V u, const V& v) {
+      const unsigned neg = (unsigned)(km >> (4 * k));
+      u.x = flip(u.x, neg);
+      u.y = flip(u.y, neg);
+      g = IM ? fma(u.y, v.x, fma(-u.x, v.y, g)) : fma(u.x, v.x, fma(u.y, v.y, g));
+    });
+    acc.add(w, g);
+  } else {  // four pairs as (t0 + e0 t1) + e1 (t2 + e0 t3) with e = +-1: no integer operation per pair
+    const T e0 = flip(T(1), (unsigned)(km >> 4)), e1 = flip(T(1), (unsigned)(km >> 8));
+    T g0 = T(0), g1 = T(0);
+    PassPairs<T, C>::run(tile, j0, xl, [&](int k, const V& u, const V& v) {
+      const T t = IM ? fma(u.y, v.x, -u.x * v.y) : fma(u.x, v.x, u.y * v.y);
+      if ((k & 3) == 0) g0 = t;
+      if ((k & 3) == 1) g0 = fma(e0, t, g0);
+      if ((k & 3) == 2) g1 = t;
+      if ((k & 3) == 3) acc.add(flip(w, (unsigned)(km >> (4 * (k & ~3)))), fma(e1, fma(e0, t, g1), g0));
+    });
+  }
+}
+
+// f(std::integral_constant<int, C>) for the group's case C.
+template <typename T, typename F>
+__device__ __forceinline__ void pass_case(int hl, F&& f) {
+  switch (hl) {
+    case 9: f(std::integral_constant<int, 1>{}); break;
+    case 10: f(std::integral_constant<int, 2>{}); break;
+    case 11: f(std::integral_constant<int, 3>{}); break;
+    case 12: f(std::integral_constant<int, PassTile<T>::S - 9>{}); break;
+    default: f(std::integral_constant<int, 0>{});
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kPassThreads, 3)
+    k_expect_pass(const typename Cx<T>::V* __restrict__ psi, int n, const ExpPass* __restrict__ passes, int npass,
+                  const PassGroup* __restrict__ groups, const PassChunk* __restrict__ chunks,
+                  const ExpChunk* __restrict__ tabs, double* partials, unsigned* counter, double* out) {
+  using V = typename Cx<T>::V;
+  constexpr int S = PassTile<T>::S, L = PassTile<T>::L, P = PassTile<T>::P, B = PassTile<T>::B;
+  constexpr unsigned E16 = 16 / sizeof(V);  // amplitudes per 16-byte copy
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  V* tile = reinterpret_cast<V*>(smem_raw);
+  __shared__ uint64_t hitab[1 << (S - L)];  // global offset of each run of 2^L amplitudes
+  __shared__ uint8_t sbits[16];
+  // the pass's groups: (xl, hl, nchunk << 19 | flags << 16 | first term's zl, chunk), the
+  // first chunk's kx[0], the first term's weight and its sign on the current tile
+  __shared__ int4 rec[kPassGroups];
+  __shared__ uint64_t signs[kPassGroups];
+  __shared__ T weight[kPassGroups];
+  __shared__ uint8_t tsign[kPassGroups];
+  const unsigned tid = threadIdx.x;
+  const int tb = n - S;
+  const uint64_t items = (uint64_t)npass << tb;
+  int cur = -1, g0 = 0, ng = 0;
+  double total = 0.0;
+  PassAcc<T> acc;
+  for (uint64_t item = blockIdx.x; item < items; item += gridDim.x) {
+    const int p = (int)(item >> tb);
+    __syncthreads();  // the last tile's readers are done
+    if (p != cur) {
+      cur = p;
+      g0 = __ldg(&passes[p].g0);
+      ng = __ldg(&passes[p].g1) - g0;
+      if (tid < 16) sbits[tid] = passes[p].sbits[tid];
+      // the groups' records: what a one-term group needs, in two 16-byte loads
+      if (tid < (unsigned)ng) {
+        const PassGroup G = groups[g0 + tid];
+        const PassChunk& C = chunks[G.chunk];
+        rec[tid] = make_int4((int)G.xl, G.hl, (G.nchunk_flags << 16) | (int)C.zl[0], G.chunk);
+        const T w = pass_weight<T>(tabs + G.chunk, 0u, (G.nchunk_flags & 2) != 0);
+        signs[tid] = C.kx[0];
+        weight[tid] = w;
+      }
+      __syncthreads();
+      for (unsigned h = tid; h < (1u << (S - L)); h += kPassThreads) {
+        uint64_t off = 0;
+#pragma unroll
+        for (int i = L; i < S; ++i) off |= (uint64_t)((h >> (i - L)) & 1u) << sbits[i];
+        hitab[h] = off;
+      }
+      __syncthreads();
+    }
+    uint64_t base = item & ((1ull << tb) - 1);
+#pragma unroll
+    for (int i = 0; i < S; ++i) base = ins0(base, sbits[i]);
+#pragma unroll 8
+    for (unsigned e = tid * E16; e < (1u << S); e += kPassThreads * E16)
+      cp_async16(tile + e, psi + (base | hitab[e >> L] | (e & ((1u << L) - 1u))));
+    if (tid < (unsigned)ng) tsign[tid] = (uint8_t)par64(__ldg(&chunks[rec[tid].w].zout[0]) & base);
+    cp_async_wait_all();
+    __syncthreads();
+    for (int g = 0; g < ng; ++g) {
+      const int4 raw = rec[g];
+      const unsigned xl = (unsigned)raw.x;
+      const int hl = raw.y, flags = (raw.z >> 16) & 7, nchunk = raw.z >> 19;
+      const unsigned j0 = hl < 0 ? tid : (unsigned)ins0(tid, hl);
+      // parity of chunk c's term t for the thread's first index in this tile
+      auto sign0 = [&](const PassChunk* C, int t) {
+        return ((unsigned)__popc(__ldg(&C->zl[t]) & j0) + par64(__ldg(&C->zout[t]) & base)) & 1u;
+      };
+      if ((flags & 4) && hl >= 0) {
+        const uint64_t km = signs[g];
+        const T w = flip(weight[g], (unsigned)__popc((unsigned)raw.z & 0xFFFFu & j0) + tsign[g]);
+        pass_case<T>(hl, [&](auto c) {
+          if (flags & 2)
+            pass_single<T, decltype(c)::value, true>(smem_raw, j0, xl, km, w, acc);
+          else
+            pass_single<T, decltype(c)::value, false>(smem_raw, j0, xl, km, w, acc);
+        });
+        continue;
+      }
+      // Re w and Im w of the thread's pairs (diagonal: |psi|^2 of its amplitudes, in
+      // two halves), then every chunk's table on them
+      for (int half = 0; half < (hl < 0 ? 2 : 1); ++half) {
+        T re[P], im[P];
+        auto pairs = [&](int k, const V& u, const V& v) {
+          re[k] = (flags & 1) ? fma(u.x, v.x, u.y * v.y) : T(0);
+          im[k] = (flags & 2) ? fma(u.y, v.x, -u.x * v.y) : T(0);
+        };
+        if (hl < 0) {
+#pragma unroll
+          for (int k = 0; k < P; ++k) {
+            const V u = tile[tid + kPassThreads * (k + half * P)];
+            pairs(k, u, u);
+          }
+        } else {
+          pass_case<T>(hl, [&](auto c) { PassPairs<T, decltype(c)::value>::run(smem_raw, j0, xl, pairs); });
+        }
+        for (int c = 0; c < nchunk; ++c) {
+          const PassChunk* C = chunks + raw.w + c;
+          const ExpChunk* W = tabs + raw.w + c;
+          unsigned i0 = 0;
+#pragma unroll
+          for (int t = 0; t < kChunkTerms; ++t) i0 |= sign0(C, t) << t;
+          const uint64_t kx = __ldg(&C->kx[half]);
+#pragma unroll
+          for (int k0 = 0; k0 < P; k0 += B) {
+            T s = T(0);
+#pragma unroll
+            for (int k = k0; k < k0 + B; ++k) {
+              const unsigned i = i0 ^ ((unsigned)(kx >> (4 * k)) & 15u);
+              if (flags & 1) s = fma(pass_weight<T>(W, i, false), re[k], s);
+              if (flags & 2) s = fma(pass_weight<T>(W, i, true), im[k], s);
+            }
+            acc.add(s);
+          }
+        }
+      }
+    }
+    total += acc.take();
+  }
+  grid_finish(total, partials, counter, out);
 }
 
 // ---------------------------------------------------------------------------
@@ -1387,6 +1632,36 @@ cudaError_t launch_expect(const void* psi, int n, qf_dtype dt, const ExpGroup* g
   prof_post(prof_slot_, s);
   count_launch();
   return cudaGetLastError();
+}
+
+template <typename T>
+static cudaError_t expect_passes_t(const void* psi, int n, const ExpPass* passes, int npass, const PassGroup* groups,
+                                   const PassChunk* chunks, const ExpChunk* tabs, double* partials, int max_blocks,
+                                   unsigned* counter, double* out, cudaStream_t s) {
+  using V = typename Cx<T>::V;
+  constexpr size_t smem = sizeof(V) << PassTile<T>::S;
+  static const cudaError_t attr =  // thread-safe one-time initialisation
+      cudaFuncSetAttribute(k_expect_pass<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (attr != cudaSuccess) return attr;
+  const uint64_t items = (uint64_t)npass << (n - PassTile<T>::S);
+  const uint64_t grid = std::min<uint64_t>({items, (uint64_t)sm_count() * 3, (uint64_t)max_blocks});
+  k_expect_pass<T><<<(unsigned)grid, kPassThreads, smem, s>>>(static_cast<const V*>(psi), n, passes, npass, groups,
+                                                              chunks, tabs, partials, counter, out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_expect_passes(const void* psi, int n, qf_dtype dt, const ExpPass* passes, int npass,
+                                 const PassGroup* groups, const PassChunk* chunks, const ExpChunk* tabs,
+                                 double* partials, int max_blocks, unsigned* counter, double* out, cudaStream_t s) {
+  if (npass <= 0 || n < (dt == QF_C128 ? PassTile<double>::S : PassTile<float>::S)) return cudaErrorInvalidValue;
+  const int prof_slot_ = prof_pre(QF_K_EXPECT, s);
+  const cudaError_t e = dt == QF_C128 ? expect_passes_t<double>(psi, n, passes, npass, groups, chunks, tabs, partials,
+                                                                max_blocks, counter, out, s)
+                                      : expect_passes_t<float>(psi, n, passes, npass, groups, chunks, tabs, partials,
+                                                               max_blocks, counter, out, s);
+  prof_post(prof_slot_, s);
+  count_launch();
+  return e;
 }
 
 cudaError_t launch_hpsi(const void* psi, void* lam, int n, qf_dtype dt, const ExpGroup* groups, int ngroups,
