@@ -242,6 +242,16 @@ struct qf_state {
   void* d_small = nullptr;
   size_t small_cap = 0;
   uint64_t small_key = 0;
+  int small_items = 0;      // items of an average block
+  // Per block of that plan: its composite at parameter t is cos(kap t) on the diagonal
+  // and s01 / s10 sin(kap t) off it, per sign class, and the generator's entry q01
+  // (closed = false: composed rotation by rotation)
+  struct SmallBlk {
+    int i, len, param;
+    bool closed;
+    double kap[4], s01[4], s10[4], q01[4];
+  };
+  std::vector<SmallBlk> small_blk;
   void* d_scoef = nullptr;
   size_t scoef_cap = 0;
   void* h_scoef = nullptr;  // page-locked
@@ -2343,6 +2353,7 @@ static qf_status energy_grad_impl(qf_state* st, uint64_t det, const qf_arot* ans
       ait = st->ansatz_plans.end();
       st->parts_key = 0;
       st->map_key = 0;
+      st->small_key = 0;
     }
   }
   // a cached plan's rotations had their masks checked when it was built
@@ -2778,6 +2789,88 @@ qf_status ensure_host(void** p, size_t* cap, size_t bytes, const char* what) {
   return QF_OK;
 }
 
+// The item map of a small sector's forward blocks (qf::SmallEval): every block's items
+// in the sweeps' order (alpha outside strings, then beta ones, both colex).
+void small_itemmap(const std::vector<qf::SecBlk>& g, const qf::SecSpace& sp, std::vector<uint2>* steps,
+                   std::vector<uint32_t>* map) {
+  steps->resize(g.size());
+  uint32_t off = 0;
+  for (size_t b = 0; b < g.size(); ++b) {
+    (*steps)[b].x = off;
+    (*steps)[b].y = g[b].cnt_e * g[b].cnt_o;
+    off += (*steps)[b].y;
+  }
+  map->resize(std::max<uint32_t>(1, off));
+  qf::HostPool::get().parallel_for(g.size(), 8, [&](size_t b) {
+    const qf::SecBlk& B = g[b];
+    // one spin's outside strings: the ranks with either pattern, and the class bits
+    struct Side { uint32_t r0, r1, cls; };
+    std::vector<Side> side[2];
+    for (int par = 0; par < 2; ++par) {
+      const uint8_t* pos = par ? B.opos : B.epos;
+      const int m = par ? B.no : B.ne, k = par ? B.ko : B.ke;
+      const uint64_t half = par ? ~kEvenMask : kEvenMask;
+      uint32_t sub = k > 0 ? (1u << k) - 1u : 0u;  // (no strings when k is outside 0..m)
+      for (uint32_t c = par ? B.cnt_o : B.cnt_e; c > 0; --c) {
+        uint64_t bits = 0;
+        for (int j = 0; j < m; ++j)
+          if ((sub >> j) & 1) bits |= 1ull << pos[j];
+        Side v{};
+        v.r0 = colex_rank(local_bits((bits | B.pat[0]) & half, par));
+        v.r1 = colex_rank(local_bits((bits | B.pat[1]) & half, par));
+        for (int j = 0; j < B.nzc; ++j) v.cls |= (uint32_t)(popc(B.zc[j] & bits) & 1) << j;
+        side[par].push_back(v);
+        if (c > 1) {  // the next k-subset in colex order
+          const uint32_t low = sub & (0u - sub), up = sub + low;
+          sub = up | (((sub ^ up) >> 2) / low);
+        }
+      }
+    }
+    uint32_t* w = map->data() + (*steps)[b].x;
+    for (const Side& e : side[0])
+      for (const Side& o : side[1])
+        *w++ = (e.r0 * sp.cnt_o + o.r0) | ((e.r1 * sp.cnt_o + o.r1) << 15) | ((e.cls ^ o.cls) << 30);
+  });
+}
+
+// A block's closed form (see compose_sparse): kap, the signed sum of its rotations'
+// coefficients per sign class, and the phases of its two active rows.  closed = false
+// when its rotations are not +-the first one there, or the composite is not real.
+void small_block(const qf_arot* ansatz, const qf_state::Blk& B, qf_state::SmallBlk* o) {
+  o->i = (int)B.i;
+  o->len = (int)(B.j - B.i);
+  o->param = ansatz[B.i].param;
+  o->closed = true;
+  const qf::SparseArgs& f = B.fwd;
+  const uint64_t x = ansatz[B.i].x;
+  const uint64_t pat[2] = {f.pat[0], f.pat[1]};
+  if ((pat[0] ^ pat[1]) != x) o->closed = false;
+  for (int c = 0; c < 4; ++c) {
+    const int cc = c < (1 << f.nzc) ? c : 0;
+    // exponent k of the phase i^k with which rotation u maps the other row onto row r
+    auto phase = [&](int u, int r) {
+      const uint64_t z = ansatz[B.i + u].z, zo = z & ~x;
+      int k = popc(x & z) + 2 * popc(z & x & pat[1 - r]);
+      for (int j = 0; j < f.nzc; ++j)
+        if (zo && zo == f.zc[j] && ((cc >> j) & 1)) k += 2;
+      return k & 3;
+    };
+    double kap = 0.0;
+    const int k0 = phase(0, 0), k1 = phase(0, 1);
+    for (int u = 0; u < o->len; ++u) {
+      const int d0 = (phase(u, 0) - k0) & 3, d1 = (phase(u, 1) - k1) & 3;
+      if (ansatz[B.i + u].x != x || ansatz[B.i + u].param != o->param || d0 != d1 || (d0 & 1)) o->closed = false;
+      kap += d0 ? -ansatz[B.i + u].coeff : ansatz[B.i + u].coeff;
+    }
+    // -i i^k is real for odd k
+    if (!(k0 & 1) || !(k1 & 1)) o->closed = false;
+    o->kap[c] = kap;
+    o->s01[c] = k0 == 1 ? 1.0 : -1.0;
+    o->s10[c] = k1 == 1 ? 1.0 : -1.0;
+    o->q01[c] = B.inv.Q[cc][0][1].y;
+  }
+}
+
 // Requests r0 .. n_req - 1 of qf_energy_grad_multi in one launch (qf::SmallEval),
 // when the handle's cached plans allow it: the ansatz and the Hamiltonian planned
 // before for this sector, every block a real two-row sector block, the direct
@@ -2815,31 +2908,51 @@ qf_status multi_small(qf_state* st, uint64_t det, const qf_arot* ansatz, size_t 
   if (qf::small_eval_smem(st->dt, members, sp.ko, sp.no) == 0) return QF_OK;
   const std::vector<qf_state::Blk>& blocks = ap.blocks;
   const size_t nblk = blocks.size();
-  for (const auto& b : blocks) {  // the reverse reads the forward geometry with the inverse's coefficients
-    if (!b.sparse || b.fwd.nr != 2 || b.inv.nr != 2 || b.fwd.nzc != b.inv.nzc) return QF_OK;
-    if (b.fwd.pat[0] != b.inv.pat[0] || b.fwd.pat[1] != b.inv.pat[1]) return QF_OK;
-    for (int j = 0; j < b.fwd.nzc; ++j)
-      if (b.fwd.zc[j] != b.inv.zc[j]) return QF_OK;
-  }
   // parameters: indices and angles of every request
   for (size_t k = 0; k < n_rot; ++k)
     if (ansatz[k].param < 0 || (size_t)ansatz[k].param >= n_par)
       return fail(QF_EINVAL, "ansatz parameter index out of range");
-  for (size_t q = r0; q < n_req; ++q)
-    for (size_t k = 0; k < n_rot; ++k)
-      if (!std::isfinite(ansatz[k].coeff * t[q * n_par + ansatz[k].param]))
-        return fail(QF_EINVAL, "theta is not finite");
+  std::atomic<bool> finite(true);
+  qf::HostPool::get().parallel_for(n_req - r0, 2, [&](size_t q) {
+    const double* tq = t + (r0 + q) * n_par;
+    bool ok = true;
+    for (size_t k = 0; k < n_rot; ++k) ok = ok && std::isfinite(ansatz[k].coeff * tq[ansatz[k].param]);
+    if (!ok) finite = false;
+  });
+  if (!finite.load()) return fail(QF_EINVAL, "theta is not finite");
   // the forward blocks' geometry for this sector, on the device once
   const uint64_t skey = content_key(nullptr, 0, ait->first ^ ((uint64_t)na << 40) ^ ((uint64_t)nbeta << 48)) | 1ull;
   if (st->small_key != skey) {
+    for (const auto& b : blocks) {  // the reverse reads the forward geometry with the inverse's coefficients
+      if (!b.sparse || b.fwd.nr != 2 || b.inv.nr != 2 || b.fwd.nzc != b.inv.nzc) return QF_OK;
+      if (b.fwd.pat[0] != b.inv.pat[0] || b.fwd.pat[1] != b.inv.pat[1]) return QF_OK;
+      for (int j = 0; j < b.fwd.nzc; ++j)
+        if (b.fwd.zc[j] != b.inv.zc[j]) return QF_OK;
+    }
     std::vector<qf::SecBlk> g(nblk);
-    for (size_t b = 0; b < nblk; ++b)
-      if (!to_secblk(blocks[b].fwd, n, na, nbeta, false, &g[b])) return QF_OK;
-    qf_status bs = ensure_buf(&st->d_small, &st->small_cap, nblk * sizeof(qf::SecBlk), "small-request blocks");
+    std::vector<qf_state::SmallBlk> sb(nblk);
+    for (size_t b = 0; b < nblk; ++b) {
+      double m[4][2][2], q[4][2][2];
+      if (!to_secblk(blocks[b].fwd, n, na, nbeta, false, &g[b]) || !sector_mq(blocks[b].inv, true, m, q)) return QF_OK;
+      small_block(ansatz, blocks[b], &sb[b]);
+    }
+    std::vector<uint2> steps;
+    std::vector<uint32_t> map;
+    small_itemmap(g, sp, &steps, &map);
+    st->small_key = 0;
+    qf_status bs = ensure_buf(&st->d_small, &st->small_cap,
+                              nblk * (sizeof(qf::SecBlk) + sizeof(uint2)) + map.size() * sizeof(uint32_t),
+                              "small-request blocks");
     if (bs != QF_OK) return bs;
-    QF_CUDA(h2d(st->d_small, g.data(), nblk * sizeof(qf::SecBlk), st->stream));
+    char* d = static_cast<char*>(st->d_small);
+    QF_CUDA(h2d(d, g.data(), nblk * sizeof(qf::SecBlk), st->stream));
+    d += nblk * sizeof(qf::SecBlk);
+    QF_CUDA(h2d(d, steps.data(), nblk * sizeof(uint2), st->stream));
+    QF_CUDA(h2d(d + nblk * sizeof(uint2), map.data(), map.size() * sizeof(uint32_t), st->stream));
     QF_CUDA(cudaStreamSynchronize(st->stream));  // g is freed on return
     st->small_key = skey;
+    st->small_items = (int)(map.size() / nblk);
+    st->small_blk.swap(sb);
   }
   qf::SecCompact cm{};
   qf_status cs = ensure_compact(st, sp, na, nbeta, &cm);
@@ -2858,39 +2971,40 @@ qf_status multi_small(qf_state* st, uint64_t det, const qf_arot* ansatz, size_t 
   std::atomic<bool> real(true);
   qf::HostPool::get().parallel_for(nr * nblk, 64, [&](size_t k) {
     const size_t q = k / nblk, b = k - q * nblk;
-    const qf_state::Blk& B = blocks[b];
+    const qf_state::SmallBlk& S = st->small_blk[b];
     const double* tq = t + (r0 + q) * n_par;
-    const int len = (int)(B.j - B.i);
-    RotIn rb_buf[16];
-    std::vector<RotIn> rb_heap;
-    RotIn* rr = rb_buf;
-    if (len > 16) {
-      rb_heap.resize(len);
-      rr = rb_heap.data();
-    }
-    for (int u = 0; u < len; ++u) {
-      const qf_arot& a = ansatz[B.i + u];
-      rr[u] = RotIn{a.x, a.z, a.coeff * tq[a.param], a.coeff};
-    }
     double m[4][2][2] = {};
-    bool ok = true;
-    compose_sparse(rr, len, false, B.fwd, [&](int c, int i, int j, cplx d) {
-      m[c][i][j] = d.real();
-      if (d.imag() != 0.0) ok = false;
-    });
-    double mi[4][2][2], qi[4][2][2];
-    if (!sector_mq(B.inv, true, mi, qi)) ok = false;
-    if (!ok) real = false;
-    const int ncls = 1 << B.fwd.nzc;
+    if (S.closed) {
+      for (int c = 0; c < 4; ++c) {
+        if (c && S.kap[c] == S.kap[c - 1] && S.s01[c] == S.s01[c - 1] && S.s10[c] == S.s10[c - 1]) {
+          std::memcpy(m[c], m[c - 1], sizeof(m[c]));
+          continue;
+        }
+        const double phi = S.kap[c] * tq[S.param], cs = std::cos(phi), sn = std::sin(phi);
+        m[c][0][0] = m[c][1][1] = cs - 1.0;
+        m[c][0][1] = S.s01[c] * sn;
+        m[c][1][0] = S.s10[c] * sn;
+      }
+    } else {
+      std::vector<RotIn> rr(S.len);
+      for (int u = 0; u < S.len; ++u) {
+        const qf_arot& a = ansatz[S.i + u];
+        rr[u] = RotIn{a.x, a.z, a.coeff * tq[a.param], a.coeff};
+      }
+      compose_sparse(rr.data(), S.len, false, blocks[b].fwd, [&](int c, int i, int j, cplx d) {
+        m[c][i][j] = d.real();
+        if (d.imag() != 0.0) real = false;
+      });
+      for (int c = 1 << blocks[b].fwd.nzc; c < 4; ++c) std::memcpy(m[c], m[0], sizeof(m[c]));
+    }
     double v[qf::kSmallCoef];
     for (int c = 0; c < 4; ++c) {
-      const int cc = c < ncls ? c : 0;
       for (int i = 0; i < 2; ++i)
         for (int j = 0; j < 2; ++j) {
-          v[4 * c + 2 * i + j] = m[cc][i][j];
-          v[16 + 4 * c + 2 * i + j] = m[cc][j][i];
+          v[4 * c + 2 * i + j] = m[c][i][j];
+          v[16 + 4 * c + 2 * i + j] = m[c][j][i];
         }
-      v[32 + c] = qi[c][0][1];
+      v[32 + c] = S.q01[c];
     }
     unsigned char* dst = static_cast<unsigned char*>(st->h_scoef) + k * rec;
     if (c128) {
@@ -2921,6 +3035,9 @@ qf_status multi_small(qf_state* st, uint64_t det, const qf_arot* ansatz, size_t 
   a.rb = cm.rb;
   a.c0 = (uint32_t)compact_of(det, sp);
   a.out = static_cast<double*>(st->d_sout);
+  a.step_threads = st->small_items;
+  a.steps = reinterpret_cast<const uint2*>(a.blks + nblk);
+  a.map = reinterpret_cast<const uint32_t*>(a.steps + nblk);
   QF_CUDA(qf::launch_small_eval(a, st->dt, (int)nr, st->stream));
   st->scale = 1.0;
   st->real = true;

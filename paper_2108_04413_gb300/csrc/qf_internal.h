@@ -440,8 +440,14 @@ struct SmallEval {
   const uint16_t* ra;
   const uint16_t* rb;  // colex rank tables of the compact layout
   uint32_t c0;         // compact index of the reference determinant
+  // Item map: block b's items are the words map[steps[b].x .. + steps[b].y), each its two
+  // members' compact indices (15 bits each) and its sign class (bits 30-31).
+  const uint32_t* map;
+  const uint2* steps;
+  int step_threads;    // a typical block's items; the launcher turns it into the steps' thread count
   double* out;         // per request: the nblk block overlaps, then <psi|H|psi> and <psi|psi>
 };
+constexpr uint32_t kSmallMaxMembers = 1u << 15;  // members an item-map word can name
 // Dynamic shared memory of one request's CTA (0 when it exceeds the limit).
 size_t small_eval_smem(qf_dtype dt, uint32_t members, int ko, int no);
 cudaError_t launch_small_eval(const SmallEval& a, qf_dtype dt, int n_req, cudaStream_t s);

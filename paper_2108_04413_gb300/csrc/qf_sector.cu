@@ -1646,64 +1646,167 @@ __global__ void __launch_bounds__(256, 4) k_sector_hpsi_direct(T* st, SecDirect 
 
 // Small systems, several requests per launch (SmallEval): CTA r evaluates request
 // r alone.  Its compact state (psi, then lambda: members real values each) and
-// the H psi step's beta-single lists live in shared memory; the block
-// geometries, tables and rank tables are shared by every CTA and stay in L1/L2.
-constexpr int kSmallThreads = 256;
+// the H psi step's beta-single lists live in shared memory; the item map and the
+// tables are shared by every CTA and stay in L1/L2.
+// A request is a chain of 2 x blocks steps, each a CTA barrier apart, so a step's
+// latency is what counts: an item's two members and class are one precomputed map
+// word instead of an unranking per item, words and coefficients are copied to a
+// ring in shared memory seven steps ahead, only as many threads as a typical block
+// has items take the steps, and the overlaps of eight steps are summed together, one
+// warp per step, exactly on the integer pipes.
+// 14 qubits, 32 requests, complex64: 965 -> 230 us, of it 55 us forward (204 steps of
+// 560 cycles), 85 us H psi (a chain of dependent lookups per member) and 87 us reverse.
+// Eight lanes per member in the H psi step, taking turns over its loops, diverged:
+// six times slower.
+constexpr int kSmallStepMax = 512;       // threads of the block steps, at most
+constexpr int kSmallRing = 8;            // steps whose map words and coefficients sit in shared memory
+constexpr int kSmallBatch = 8;           // steps whose overlaps are summed together
+constexpr size_t kSmallSmemMax = 200u * 1024u;  // psi, lambda and the beta-single lists of 256 threads
+constexpr size_t kSmallSmemCap = 224u * 1024u;  // with all else (static shared memory: under 3 KB of 227)
 
-// The two compact indices and the sign class of item `it` of block B (the item's
-// outside string in colex order, as the full-layout sweep enumerates it).
-__device__ __forceinline__ void small_item(const SecBlk& B, uint32_t it, const uint32_t (*C)[kBinom],
-                                           const uint16_t* __restrict__ ra, const uint16_t* __restrict__ rb,
-                                           uint32_t cnt_o, uint32_t* i0, uint32_t* i1, unsigned* cls) {
-  const uint32_t ie = it / B.cnt_o, io = it - ie * B.cnt_o;
-  const uint64_t base = unrank(ie, B.epos, B.ne, B.ke, C) | unrank(io, B.opos, B.no, B.ko, C);
-  unsigned c = 0;
-  if (B.nzc > 0) c = par64s(B.zc[0] & base);
-  if (B.nzc > 1) c |= par64s(B.zc[1] & base) << 1;
-  const uint32_t q0 = (uint32_t)(base | B.pat[0]), q1 = (uint32_t)(base | B.pat[1]);
-  *i0 = (uint32_t)__ldg(ra + gather_even(q0)) * cnt_o + __ldg(rb + gather_even(q0 >> 1));
-  *i1 = (uint32_t)__ldg(ra + gather_even(q1)) * cnt_o + __ldg(rb + gather_even(q1 >> 1));
-  *cls = c;
+// Asynchronous copy of one 4- or 8-byte value to shared memory.
+template <typename T> __device__ __forceinline__ void cp_async_small(T* smem, const T* gmem) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(a), "l"(gmem), "n"(sizeof(T)) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kSmallThreads, 2) k_small_eval(SmallEval a) {
+// FP32 values are summed exactly as float pairs (TwoSum), FP64 ones in FP64.
+template <typename T> struct StepSum;
+template <> struct StepSum<double> {
+  double v = 0.0;
+  __device__ __forceinline__ void add(double d) { v += d; }
+  __device__ __forceinline__ void add(const StepSum& o) { v += o.v; }
+  __device__ __forceinline__ long long warp(int* e) const { return warp_sum_fixed(v, e); }
+};
+template <> struct StepSum<float> {
+  float2 v = make_float2(0.f, 0.f);
+  __device__ __forceinline__ void add(float d) {
+    float e;
+    v.x = two_sum(v.x, d, &e);
+    v.y = __fadd_rn(v.y, e);
+  }
+  __device__ __forceinline__ void add(const StepSum& o) {
+    add(o.v.x);
+    v.y = __fadd_rn(v.y, o.v.y);
+  }
+  __device__ __forceinline__ long long warp(int* e) const {
+    float2 r;  // normalised: the low part below the high part's last bit
+    r.x = two_sum(v.x, v.y, &r.y);
+    return warp_sum_fixed_ds(r, e);
+  }
+};
+
+// Barrier of the CTA's first n threads (whole warps).
+__device__ __forceinline__ void step_barrier(int n) { asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory"); }
+
+// Dynamic shared memory: psi and lambda, the map words of kSmallRing steps (two per
+// step thread), the overlaps of kSmallBatch steps (each step thread's), then the H psi
+// step's beta-single lists, which share the room of the two before (the sweeps come
+// before and after it).
+template <typename T, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_small_eval(SmallEval a) {
+  const int ST = a.step_threads, NW = ST / 32;  // threads and warps of the block steps
   extern __shared__ __align__(16) unsigned char dsm[];
   __shared__ uint32_t C[kBinom][kBinom];
-  const int tid = threadIdx.x;
+  __shared__ T cw[kSmallRing][20];  // the coefficients of the coming steps
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t M = a.cnt_e * a.cnt_o;
+  const int nb = a.nblk;
   T* ps = reinterpret_cast<T*>(dsm);
   T* lm = ps + M;
-  uint32_t* bsl = reinterpret_cast<uint32_t*>(dsm + align16(2 * (size_t)M * sizeof(T)));
+  uint16_t* sn = reinterpret_cast<uint16_t*>(dsm + align16(2 * (size_t)M * sizeof(T)));  // every block's items
+  unsigned char* room = reinterpret_cast<unsigned char*>(sn) + align16(nb * sizeof(uint16_t));
+  uint32_t* mw = reinterpret_cast<uint32_t*>(room);
+  StepSum<T>* red = reinterpret_cast<StepSum<T>*>(mw + kSmallRing * 2 * ST);
+  uint32_t* bsl = reinterpret_cast<uint32_t*>(room);
   const T* cf = static_cast<const T*>(a.coef) + (size_t)blockIdx.x * a.nblk * kSmallCoef;
   double* out = a.out + (size_t)blockIdx.x * (a.nblk + 2);
   fill_binom(C);
-  for (uint32_t m = tid; m < M; m += kSmallThreads) ps[m] = (m == a.c0) ? T(1) : T(0);
+  for (int b = tid; b < nb; b += NT) sn[b] = (uint16_t)__ldg(&a.steps[b].y);
+  for (uint32_t m = tid; m < M; m += NT) ps[m] = (m == a.c0) ? T(1) : T(0);
+  // the block steps in order (REV: from the last block, with the inverse's
+  // coefficients and the overlaps); item(i0, i1, m, class, sum) handles one item
+  auto sweep = [&](auto rev, auto&& item) {
+    constexpr bool REV = decltype(rev)::value;
+    constexpr int NC = REV ? 20 : 16;  // mi then q, or m
+    constexpr int D = kSmallRing - 1;  // steps loaded ahead
+    auto blk = [&](int s) { return REV ? nb - 1 - s : s; };
+    // map offsets of the step to load and of the current step
+    uint32_t lo = 0, so = 0;
+    if (REV && nb > 0) lo = so = __ldg(&a.steps[nb - 1].x) + sn[nb - 1];
+    auto load = [&](int s) {  // one step's loads are one copy group
+      if (s < nb) {
+        const int slot = s & (kSmallRing - 1);
+        const uint32_t n = sn[blk(s)];
+        if (REV) lo -= n;
+        uint32_t* w = mw + slot * 2 * ST + tid;
+        if ((uint32_t)tid < n) cp_async_small(w, a.map + lo + tid);
+        if ((uint32_t)(tid + ST) < n) cp_async_small(w + ST, a.map + lo + tid + ST);
+        if (tid < NC) cp_async_small(&cw[slot][tid], cf + (size_t)blk(s) * kSmallCoef + (REV ? 16 : 0) + tid);
+        if (!REV) lo += n;
+      }
+      cp_async_commit();
+    };
+    for (int s = 0; s < D; ++s) load(s);
+    cp_async_wait<D - 1>();
+    step_barrier(ST);
+    // sums of the last `cnt` steps before step s, a warp per step
+    auto reduce = [&](int s, int cnt) {
+      for (int r = warp; r < cnt; r += NW) {
+        const int q = s - cnt + r;
+        const StepSum<T>* row = red + (q & (2 * kSmallBatch - 1)) * ST;
+        const uint32_t n = sn[blk(q)];
+        StepSum<T> v;
+        for (uint32_t j = lane; j < (uint32_t)ST && (j & ~31u) < n; j += 32) v.add(row[j]);
+        int e;
+        const long long t = v.warp(&e);
+        const double d = warp_fixed_to_double(lane == 0 ? t : 0ll, lane == 0 ? e : 0);
+        if (lane == 0) out[blk(q)] = d;
+      }
+    };
+    for (int s = 0; s < nb; ++s) {
+      const int slot = s & (kSmallRing - 1);
+      load(s + D);  // into the slot of step s - 1
+      const uint32_t n = sn[blk(s)];
+      if (REV) so -= n;
+      const T* c = cw[slot];
+      StepSum<T> acc;
+      for (uint32_t it = tid; it < n; it += (uint32_t)ST) {
+        const uint32_t w = it < 2u * ST ? mw[slot * 2 * ST + it] : __ldg(a.map + so + it);
+        item(w & 0x7FFFu, (w >> 15) & 0x7FFFu, c, w >> 30, acc);
+      }
+      if (REV && (uint32_t)(tid & ~31) < n) red[(s & (2 * kSmallBatch - 1)) * ST + tid] = acc;
+      if (!REV) so += n;
+      cp_async_wait<D - 1>();  // step s + 1 is there
+      step_barrier(ST);
+      // the rows of a finished batch are rewritten only after the next batch's steps
+      if (REV && ((s + 1) & (kSmallBatch - 1)) == 0) reduce(s + 1, kSmallBatch);
+    }
+    cp_async_wait<0>();
+    if (REV) reduce(nb, nb & (kSmallBatch - 1));
+  };
   __syncthreads();
-  // forward: psi <- psi + (M - I) psi on every item of each block in turn
-  for (int b = 0; b < a.nblk; ++b) {
-    const SecBlk& B = a.blks[b];
-    const T* mf = cf + (size_t)b * kSmallCoef;
-    const uint32_t items = B.cnt_e * B.cnt_o;
-    for (uint32_t it = tid; it < items; it += kSmallThreads) {
-      uint32_t i0, i1;
-      unsigned cls;
-      small_item(B, it, C, a.ra, a.rb, a.cnt_o, &i0, &i1, &cls);
-      const T* m = mf + 4 * cls;
+  // forward: psi <- psi + (M - I) psi
+  if (tid < ST) {
+    sweep(std::false_type{}, [&](uint32_t i0, uint32_t i1, const T* c, uint32_t cls, StepSum<T>&) {
+      const T* m = c + 4 * cls;
       const T v0 = ps[i0], v1 = ps[i1];
       ps[i0] = fma(m[0], v0, fma(m[1], v1, v0));
       ps[i1] = fma(m[2], v0, fma(m[3], v1, v1));
-    }
-    __syncthreads();
+    });
   }
+  __syncthreads();
   // lambda = H psi with <psi|lambda> and <psi|psi>
   double acc_e = 0.0, acc_n = 0.0;
   auto amp = [&](size_t m) -> double { return (double)ps[m]; };
   auto pair_op = [&](size_t m) { return ps[m]; };
-  for (uint32_t m = tid; m < M; m += kSmallThreads) {
+  for (uint32_t m = tid; m < M; m += NT) {
+    const double lx = direct_member<T, false, NT>(m, a.d, a.cnt_o, a.ke, a.ko, a.ra, a.rb, C, bsl + tid, amp, pair_op);
     const double self = (double)ps[m];
-    const double lx = direct_member<T, false, kSmallThreads>(m, a.d, a.cnt_o, a.ke, a.ko, a.ra, a.rb, C, bsl + tid,
-                                                             amp, pair_op);
     lm[m] = (T)lx;
     acc_e = fma(self, lx, acc_e);
     acc_n = fma(self, self, acc_n);
@@ -1711,36 +1814,34 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small_eval(SmallEval a) {
   acc_e = block_sum_s(acc_e);
   acc_n = block_sum_s(acc_n);
   if (tid == 0) {
-    out[a.nblk] = acc_e;
-    out[a.nblk + 1] = acc_n;
+    out[nb] = acc_e;
+    out[nb + 1] = acc_n;
   }
-  __syncthreads();
   // reverse: block b's overlap Im <lambda|Q_b|psi> = q01 (lambda0 psi1 - lambda1 psi0)
   // summed over its items, then psi and lambda un-rotated by its inverse
-  for (int b = a.nblk - 1; b >= 0; --b) {
-    const SecBlk& B = a.blks[b];
-    const T* mi = cf + (size_t)b * kSmallCoef + 16;
-    const T* q = cf + (size_t)b * kSmallCoef + 32;
-    const uint32_t items = B.cnt_e * B.cnt_o;
-    double acc = 0.0;
-    for (uint32_t it = tid; it < items; it += kSmallThreads) {
-      uint32_t i0, i1;
-      unsigned cls;
-      small_item(B, it, C, a.ra, a.rb, a.cnt_o, &i0, &i1, &cls);
-      const T* m = mi + 4 * cls;
-      const T p0 = ps[i0], p1 = ps[i1], w0 = lm[i0], w1 = lm[i1];
-      acc += (double)(q[cls] * fma(w0, p1, -w1 * p0));
-      ps[i0] = fma(m[0], p0, fma(m[1], p1, p0));
-      ps[i1] = fma(m[2], p0, fma(m[3], p1, p1));
-      lm[i0] = fma(m[0], w0, fma(m[1], w1, w0));
-      lm[i1] = fma(m[2], w0, fma(m[3], w1, w1));
-    }
-    acc = block_sum_s(acc);  // its first barrier also ends this block's updates
-    if (tid == 0) out[b] = acc;
-  }
+  __syncthreads();
+  if (tid < ST) sweep(std::true_type{}, [&](uint32_t i0, uint32_t i1, const T* c, uint32_t cls, StepSum<T>& acc) {
+    const T* m = c + 4 * cls;
+    const T p0 = ps[i0], p1 = ps[i1], l0 = lm[i0], l1 = lm[i1];
+    acc.add(c[16 + cls] * fma(l0, p1, -l1 * p0));
+    ps[i0] = fma(m[0], p0, fma(m[1], p1, p0));
+    ps[i1] = fma(m[2], p0, fma(m[3], p1, p1));
+    lm[i0] = fma(m[0], l0, fma(m[1], l1, l0));
+    lm[i1] = fma(m[2], l0, fma(m[3], l1, l1));
+  });
 }
 
 }  // namespace
+
+static int sm_count_s() {
+  static const int v = [] {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return std::max(1, sms);
+  }();
+  return v;
+}
 
 // Grid of the cooperative sweep: about one item per thread for a typical block,
 // at most one CTA per SM (all CTAs must be resident at once; a 1024-thread CTA
@@ -2074,34 +2175,55 @@ cudaError_t launch_sector_hpsi(const void* psi, void* lam, qf_dtype dt, bool rea
   return e;
 }
 
+// Bytes of psi, lambda and the beta-single lists of 256 threads.
 size_t small_eval_smem(qf_dtype dt, uint32_t members, int ko, int no) {
   const size_t real = dt == QF_C128 ? sizeof(double) : sizeof(float);
-  const size_t b = align16(2 * (size_t)members * real) +
-                   (size_t)std::max(1, ko * (no - ko)) * kSmallThreads * sizeof(uint32_t);
-  return b <= 200u * 1024u ? b : 0;
+  const size_t b = align16(2 * (size_t)members * real) + (size_t)std::max(1, ko * (no - ko)) * 256 * sizeof(uint32_t);
+  return members < kSmallMaxMembers && b <= kSmallSmemMax ? b : 0;
 }
 
-cudaError_t launch_small_eval(const SmallEval& a, qf_dtype dt, int n_req, cudaStream_t s) {
-  if (n_req <= 0 || a.nblk < 0) return cudaSuccess;
-  const size_t smem = small_eval_smem(dt, a.cnt_e * a.cnt_o, a.ko, a.d.no);
-  if (smem == 0 || a.d.n > 32 || a.cnt_o > (1u << 14)) return cudaErrorInvalidValue;
-  const auto k = dt == QF_C128 ? k_small_eval<double> : k_small_eval<float>;
-  static std::once_flag once_d, once_f;  // allow the opt-in shared memory size, once per process
-  static cudaError_t attr_d = cudaSuccess, attr_f = cudaSuccess;
-  if (dt == QF_C128)
-    std::call_once(once_d, [&] {
-      attr_d = cudaFuncSetAttribute(k_small_eval<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    });
-  else
-    std::call_once(once_f, [&] {
-      attr_f = cudaFuncSetAttribute(k_small_eval<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    });
-  const cudaError_t attr = dt == QF_C128 ? attr_d : attr_f;
+template <typename T, int NT>
+static cudaError_t small_eval_t(const SmallEval& a, int n_req, size_t smem, cudaStream_t s) {
+  static const cudaError_t attr =  // allow the opt-in shared memory size, once per process
+      cudaFuncSetAttribute(k_small_eval<T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmemCap);
   if (attr != cudaSuccess) return attr;
+  k_small_eval<T, NT><<<n_req, NT, smem, s>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_small_eval(const SmallEval& req, qf_dtype dt, int n_req, cudaStream_t s) {
+  if (n_req <= 0 || req.nblk < 0) return cudaSuccess;
+  SmallEval a = req;
+  const uint32_t members = a.cnt_e * a.cnt_o;
+  if (small_eval_smem(dt, members, a.ko, a.d.no) == 0 || a.d.n > 32 || a.cnt_o > (1u << 14) || !a.map)
+    return cudaErrorInvalidValue;
+  // H psi by 1024 threads while every request has an SM to itself, else 512, so that
+  // two requests share one; 256 where the lists need the room.  The steps by as many
+  // as a typical block has items (a step's fixed work grows with its warps).
+  const size_t real = dt == QF_C128 ? sizeof(double) : sizeof(float);
+  const size_t fixed = align16(2 * (size_t)members * real) + align16(a.nblk * sizeof(uint16_t));
+  int nt = n_req <= sm_count_s() ? 1024 : 512;
+  size_t smem = 0;
+  for (;; nt /= 2) {
+    const size_t lists = (size_t)std::max(1, a.ko * (a.d.no - a.ko)) * nt * sizeof(uint32_t);
+    for (a.step_threads = std::min({nt, kSmallStepMax, std::max(128, (req.step_threads + 127) / 128 * 128)});;
+         a.step_threads -= 32) {
+      const size_t steps = (size_t)a.step_threads * (kSmallRing * 2 * sizeof(uint32_t) + kSmallBatch * 2 * 8);
+      smem = fixed + std::max(lists, steps);
+      if (smem <= kSmallSmemCap || a.step_threads == 96) break;
+    }
+    if (smem <= kSmallSmemCap || nt == 256) break;
+  }
+  if (smem > kSmallSmemCap) return cudaErrorInvalidValue;
   const int prof_slot_ = prof_pre(QF_K_SPARSE, s);
-  k<<<n_req, kSmallThreads, smem, s>>>(a);
+  const cudaError_t e =
+      dt == QF_C128 ? (nt == 1024  ? small_eval_t<double, 1024>(a, n_req, smem, s)
+                       : nt == 512 ? small_eval_t<double, 512>(a, n_req, smem, s)
+                                   : small_eval_t<double, 256>(a, n_req, smem, s))
+                    : (nt == 1024  ? small_eval_t<float, 1024>(a, n_req, smem, s)
+                       : nt == 512 ? small_eval_t<float, 512>(a, n_req, smem, s)
+                                   : small_eval_t<float, 256>(a, n_req, smem, s));
   count_launch();
-  const cudaError_t e = cudaGetLastError();
   prof_post(prof_slot_, s);
   return e;
 }
