@@ -1687,6 +1687,10 @@ bool build_runs(const qf::SecBlk* sec, size_t nblk, int n, int na, int nb, uint6
     R.b1 = (int)b1;
     R.ua = ua;
     R.ub = ub;
+    R.ne = ne;
+    R.no = no;
+    R.na = na;
+    R.nb = nb;
     int loca[32] = {0}, locb[32] = {0};  // spin-local orbital -> run-local index
     uint32_t Ga = 0, Gb = 0;             // spin-local masks of G
     {

@@ -250,6 +250,7 @@ struct RunInfo {
   int ua, ub;
   uint8_t apos[kSecMaxPos], bpos[kSecMaxPos];  // spin-local orbital of each run-local index
   uint32_t maxsize;                 // largest part
+  int ne, no, na, nb;               // the sector: alpha / beta orbitals and electrons
 };
 
 // Compact sector layout: member (alpha string a, beta string b), both as local
@@ -396,7 +397,7 @@ cudaError_t launch_sector_runs(void* psi, void* lam, qf_dtype dt, bool adj, bool
                                const uint32_t* map, bool ds, bool dss, cudaStream_t s);
 // Overlaps only: out[b] = Im <lam|Q_b|psi> of every block b on the same compact
 // state (psi real parts, lam real parts in psi's imaginary slots); nothing is
-// rotated.  Same descriptors as launch_sector_runs.
+// rotated.  Same descriptors as launch_sector_runs; partial holds nblk * pmax values.
 cudaError_t launch_sector_overlaps(void* psi, qf_dtype dt, const RunInfo* runs, int nruns, const RunPart* parts,
                                   const RunBlk* blks, int nblk, double* partial, int pmax, double* out,
                                   const SecCompact& cm, const uint16_t* strs, cudaStream_t s);

@@ -407,11 +407,10 @@ static_assert(sizeof(RunBlk) % 4 == 0 && kRunBlkWords <= kRunThreads && kRunBlkW
 // Shared-memory bytes per member: psi real parts (forward), (psi, lam) packed
 // real pairs (reverse, real), psi and lam complex (reverse, complex), or lam's
 // real parts (reverse, real, psi read from the forward log); plus the member's
-// compact index, kept for the scatter (the read-only MODE 4 has none).
+// compact index, kept for the scatter.
 template <int MODE, typename T>
 __host__ __device__ constexpr size_t run_member_bytes() {
-  return (MODE == 0 || MODE == 3 ? sizeof(T) : (MODE == 1 || MODE == 4) ? 2 * sizeof(T) : 4 * sizeof(T)) +
-         (MODE == 4 ? 0 : sizeof(uint32_t));
+  return (MODE == 0 || MODE == 3 ? sizeof(T) : MODE == 1 ? 2 * sizeof(T) : 4 * sizeof(T)) + sizeof(uint32_t);
 }
 __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~(size_t)15; }
 
@@ -426,8 +425,6 @@ __device__ void fill_binom_prefix(uint32_t (*Cs)[kBinom]) {
 // MODE 2: reverse, psi and lam complex.
 // MODE 3: reverse, lam real (psi's imaginary slots); psi after each block is
 // read back from the forward log instead of being un-rotated.
-// MODE 4: overlaps only, psi and lam real and packed: every block's overlap on
-// the same (psi, lam), nothing rotated or written back (operator-pool gradients).
 // Overlaps accumulate in the state's precision (FP64 for complex128, FP32 for
 // complex64); each part's overlap with a block is written to partial in FP64.
 // Programmatic dependent launch: a sweep launch may start while the previous
@@ -477,9 +474,9 @@ __device__ __forceinline__ void sector_run_body(typename SCx<T>::V* psi, typenam
   const uint32_t cap = R.maxsize;
   T* ar = reinterpret_cast<T*>(dsm);   // MODE 0 (psi), MODE 3 (lam)
   float2* ad = reinterpret_cast<float2*>(dsm);  // the same, double-single (DSW)
-  V* av = reinterpret_cast<V*>(dsm);   // MODE 1, 2, 4 (psi)
+  V* av = reinterpret_cast<V*>(dsm);   // MODE 1, 2 (psi)
   V* lv = av + cap;                    // MODE 2 (lam)
-  constexpr size_t idx_bytes = MODE == 4 ? 0 : sizeof(uint32_t);
+  constexpr size_t idx_bytes = sizeof(uint32_t);
   const size_t amp_bytes = align16((run_member_bytes<MODE, T>() - idx_bytes) * cap);
   uint32_t* gi = reinterpret_cast<uint32_t*>(dsm + amp_bytes);
   const uint32_t size = P.cnta * P.cntb;
@@ -529,7 +526,7 @@ __device__ __forceinline__ void sector_run_body(typename SCx<T>::V* psi, typenam
     const uint32_t sa = unrank_m(ia, R.apos, R.ua, P.ka, C) | P.ga;
     const uint32_t sbm = unrank_m(ib, R.bpos, R.ub, P.kb, C) | P.gb;
     const uint32_t g = (uint32_t)compact_index(cm, sa, sbm);
-    if (MODE != 4) gi[m] = g;
+    gi[m] = g;
     if (DSW) {  // double-single state layout (dss): the slot already holds the (hi, lo) pair
       ad[m] = dss ? __ldcg(reinterpret_cast<const float2*>(psi) + 2 * (size_t)g + slot)
                   : ds_of(__ldcg(pr + 2 * (size_t)g + slot));
@@ -780,9 +777,6 @@ __device__ __forceinline__ void sector_run_body(typename SCx<T>::V* psi, typenam
           acc = fma(q01, fma(w0, pp.y, -w1 * pp.x), acc);
           ar[i0] = fma(a00, w0, fma(a01, w1, w0));
           ar[i1] = fma(a10, w0, fma(a11, w1, w1));
-        } else if (MODE == 4) {
-          const V p0 = av[i0], p1 = av[i1];  // (psi, lambda)
-          acc = fma(q01, fma(p0.y, p1.x, -p1.y * p0.x), acc);
         } else if (MODE == 1) {
           const V p0 = av[i0], p1 = av[i1];  // (psi, lambda)
           // Im <lam|Q|psi> on the pair, Qi = [[0, q01], [-q01, 0]] (checked on the host)
@@ -840,7 +834,6 @@ __device__ __forceinline__ void sector_run_body(typename SCx<T>::V* psi, typenam
   // the next run may launch once every CTA is here (its CTAs then take the SMs as
   // this run's scatters finish, so that they spread over the SMs)
   grid_dep_launch_dependents();
-  if (MODE == 4) return;  // read only
   T* pw = reinterpret_cast<T*>(psi);
   for (uint32_t m = tid; m < size; m += NT) {
     const uint32_t g = gi[m];
@@ -913,6 +906,116 @@ __global__ void __launch_bounds__(kRunThreads) k_run_itemmap(RunInfo run, const 
     }
     off += items;
   }
+}
+
+// Operator-pool overlaps (nothing is rotated, so no block waits for another): CTA
+// (block, slice) takes the block's whole sector at once, a slice of its outside alpha
+// strings against every outside beta string.  Each string's rank with either pattern
+// and its class bits are listed in shared memory once, so an item is two listed words,
+// two members and one product.  Bound by the members' reads from L2 (32 bytes per
+// item) and, in complex128, three FP64 operations per item.
+// 20 qubits, pool of 875 operators (4.4 M items), complex128: 1290 us as part-local
+// runs with a CTA barrier per block, 47 us here.
+constexpr int kPoolRuns = 40;  // runs described by one launch (kernel arguments stay under 4 KB)
+struct PoolRuns {
+  int n, slices;
+  RunInfo run[kPoolRuns];
+};
+template <typename T>
+__global__ void __launch_bounds__(256) k_pool_overlaps(const typename SCx<T>::V* __restrict__ psi,
+                                                       const RunBlk* __restrict__ blks, double* partial,
+                                                       SecCompact cm, const __grid_constant__ PoolRuns pr) {
+  using V = typename SCx<T>::V;
+  extern __shared__ __align__(16) unsigned char dsm[];
+  __shared__ uint32_t C[kBinom][kBinom];
+  __shared__ uint8_t pos[2][kSecMaxPos];         // outside orbitals of each spin
+  __shared__ uint32_t pat[2][2], zm[2][2], cnt[2];  // spin-local patterns [i][spin], class masks [j][spin]
+  __shared__ int el[2], m[2];                    // electrons outside, outside orbitals
+  __shared__ T q[kSparseMaxCls];
+  const int tid = threadIdx.x;
+  const int b = pr.run[0].b0 + (int)blockIdx.x / pr.slices, slice = (int)blockIdx.x % pr.slices;
+  int r = 0;
+  while (b >= pr.run[r].b1) ++r;  // uniform over the CTA
+  const RunInfo& R = pr.run[r];
+  const RunBlk& B = blks[b];
+  fill_binom(C);
+  if (tid < 2) {  // one thread per spin
+    const int u = tid ? R.ub : R.ua, orb = tid ? R.no : R.ne;
+    const uint8_t* loc = tid ? R.bpos : R.apos;
+    const uint8_t* out = tid ? B.opos : B.epos;
+    const int nout = tid ? B.no : B.ne;
+    uint32_t local_out = 0, supp = 0;
+    for (int i = 0; i < nout; ++i) local_out |= 1u << out[i];
+    uint32_t p0 = 0, p1 = 0, z0 = B.zg[0][tid], z1 = B.zg[1][tid];
+    for (int i = 0; i < u; ++i) {
+      const uint32_t bit = 1u << loc[i];
+      if (!((local_out >> i) & 1u)) supp |= bit;
+      if ((B.pu[0][tid] >> i) & 1u) p0 |= bit;
+      if ((B.pu[1][tid] >> i) & 1u) p1 |= bit;
+      if ((B.zu[0][tid] >> i) & 1u) z0 |= bit;
+      if ((B.zu[1][tid] >> i) & 1u) z1 |= bit;
+    }
+    int k = 0;
+    for (int i = 0; i < orb; ++i)
+      if (!((supp >> i) & 1u)) pos[tid][k++] = (uint8_t)i;
+    m[tid] = k;
+    el[tid] = (tid ? R.nb : R.na) - (tid ? B.o0 : B.e0);
+    pat[0][tid] = p0;
+    pat[1][tid] = p1;
+    zm[0][tid] = B.nzc > 0 ? z0 : 0u;
+    zm[1][tid] = B.nzc > 1 ? z1 : 0u;
+  }
+  if (tid < kSparseMaxCls) q[tid] = sizeof(T) == 8 ? (T)B.q[tid][0][1] : (T)B.qf[tid];
+  __syncthreads();
+  if (tid < 2) cnt[tid] = (el[tid] >= 0 && el[tid] <= m[tid]) ? C[m[tid]][el[tid]] : 0u;
+  __syncthreads();
+  // rank with pattern 0 | rank with pattern 1 << 15 | class bits << 30
+  const uint32_t per = (cnt[0] + pr.slices - 1) / pr.slices, a0 = min(cnt[0], slice * per);
+  const uint32_t na = min(cnt[0], a0 + per) - a0, nb = cnt[1];
+  uint32_t* lb = reinterpret_cast<uint32_t*>(dsm);
+  uint32_t* la = lb + nb;
+  auto entry = [&](uint32_t i, int spin) {
+    const uint32_t s = unrank_m(i, pos[spin], m[spin], el[spin], C);
+    const uint16_t* rk = spin ? cm.rb : cm.ra;
+    return (uint32_t)__ldg(rk + (s | pat[0][spin])) | ((uint32_t)__ldg(rk + (s | pat[1][spin])) << 15) |
+           (par32s(zm[0][spin] & s) << 30) | (par32s(zm[1][spin] & s) << 31);
+  };
+  if (na > 0 && nb > 0) {
+    for (uint32_t i = tid; i < nb; i += 256) lb[i] = entry(i, 1);
+    for (uint32_t i = tid; i < na; i += 256) la[i] = entry(a0 + i, 0);
+  }
+  __syncthreads();
+  double acc = 0.0;
+  const uint64_t items = (uint64_t)na * nb;
+  if (items) {
+    uint32_t ia = tid / nb, ib = tid % nb;
+    const uint32_t da = 256 / nb, db = 256 % nb;
+    for (uint64_t it = tid; it < items; it += 256) {
+      const uint32_t wa = la[ia], wb = lb[ib];
+      const size_t i0 = (size_t)(wa & 0x7FFFu) * cm.cnt_o + (wb & 0x7FFFu);
+      const size_t i1 = (size_t)((wa >> 15) & 0x7FFFu) * cm.cnt_o + ((wb >> 15) & 0x7FFFu);
+      const V p0 = __ldg(psi + i0), p1 = __ldg(psi + i1);  // (psi, lambda)
+      // Im <lam|Q|psi> on the pair, Qi = [[0, q01], [-q01, 0]] (checked on the host)
+      acc += (double)(q[(wa ^ wb) >> 30] * fma(p0.y, p1.x, -p1.y * p0.x));
+      ia += da;
+      ib += db;
+      if (ib >= nb) {
+        ib -= nb;
+        ++ia;
+      }
+    }
+  }
+  acc = block_sum_s(acc);
+  if (tid == 0) partial[(size_t)b * pr.slices + slice] = acc;
+}
+
+// out[b] = the sum of block b's slices, in order.
+__global__ void k_pool_reduce(const double* __restrict__ partial, int slices, int nblk, double* out) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= nblk) return;
+  double s = 0.0;
+  for (int k = 0; k < slices; ++k) s += partial[(size_t)b * slices + k];
+  out[b] = s;
 }
 
 // out[b] = sum over the parts of block b's run of partial[b * pmax + part], in part order.
@@ -1907,7 +2010,7 @@ static size_t run_smem_max() {
 
 template <int MODE, typename T>
 static size_t run_smem_bytes(uint32_t maxsize) {
-  constexpr size_t idx = MODE == 4 ? 0 : sizeof(uint32_t);
+  constexpr size_t idx = sizeof(uint32_t);
   const size_t amp = align16((run_member_bytes<MODE, T>() - idx) * maxsize);
   return align16(amp + idx * maxsize);
 }
@@ -2032,20 +2135,43 @@ cudaError_t launch_run_itemmaps(const RunInfo* runs, int nruns, const RunPart* p
   return cudaSuccess;
 }
 
-cudaError_t launch_sector_overlaps(void* psi, qf_dtype dt, const RunInfo* runs, int nruns, const RunPart* parts,
+// Slices of a block's alpha strings: enough CTAs for eight per SM, within the partials.
+template <typename T>
+static cudaError_t overlaps_t(const void* psi, const RunInfo* runs, int nruns, const RunBlk* blks, int nblk,
+                              double* partial, int pmax, double* out, const SecCompact& cm, cudaStream_t s) {
+  using V = typename SCx<T>::V;
+  constexpr int kMaxLists = 200 * 1024;  // the largest sector's strings: 2 x C(17, 8) words = 194480 bytes
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(k_pool_overlaps<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxLists);
+  if (attr != cudaSuccess) return attr;
+  PoolRuns pr;
+  pr.slices = std::max(1, std::min(pmax, 8 * sm_count_s() / std::max(1, nblk)));
+  uint64_t cnt_e = 1;  // C(ne, na) >= any block's outside alpha strings
+  for (int k = 1; k <= runs[0].na; ++k) cnt_e = cnt_e * (uint64_t)(runs[0].ne - runs[0].na + k) / k;
+  const size_t smem = (cm.cnt_o + (cnt_e + pr.slices - 1) / pr.slices) * sizeof(uint32_t);
+  if (smem > (size_t)kMaxLists) return cudaErrorInvalidValue;
+  for (int r0 = 0; r0 < nruns; r0 += kPoolRuns) {
+    pr.n = std::min(kPoolRuns, nruns - r0);
+    std::copy(runs + r0, runs + r0 + pr.n, pr.run);
+    const int nb = pr.run[pr.n - 1].b1 - pr.run[0].b0;
+    k_pool_overlaps<T><<<nb * pr.slices, 256, smem, s>>>(static_cast<const V*>(psi), blks, partial, cm, pr);
+    count_launch();
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  k_pool_reduce<<<(nblk + 255) / 256, 256, 0, s>>>(partial, pr.slices, nblk, out);
+  count_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_sector_overlaps(void* psi, qf_dtype dt, const RunInfo* runs, int nruns, const RunPart*,
                                   const RunBlk* blks, int nblk, double* partial, int pmax, double* out,
-                                  const SecCompact& cm, const uint16_t* strs, cudaStream_t s) {
+                                  const SecCompact& cm, const uint16_t*, cudaStream_t s) {
   if (nblk <= 0 || nruns <= 0) return cudaSuccess;
   if (!cm.ra) return cudaErrorInvalidValue;
   const int prof_slot_ = prof_pre(QF_K_ADJ_SPARSE, s);
-  cudaError_t e = (dt == QF_C128)
-                      ? runs_t<4, double>(psi, psi, runs, nruns, parts, blks, partial, pmax, cm, nullptr, strs, nullptr, false, s)
-                      : runs_t<4, float>(psi, psi, runs, nruns, parts, blks, partial, pmax, cm, nullptr, strs, nullptr, false, s);
-  if (e == cudaSuccess) {
-    k_sector_reduce_parts<<<(nblk + 7) / 8, 256, 0, s>>>(partial, pmax, blks, nblk, out);
-    e = cudaGetLastError();
-    count_launch();
-  }
+  const cudaError_t e = dt == QF_C128 ? overlaps_t<double>(psi, runs, nruns, blks, nblk, partial, pmax, out, cm, s)
+                                      : overlaps_t<float>(psi, runs, nruns, blks, nblk, partial, pmax, out, cm, s);
   prof_post(prof_slot_, s);
   return e;
 }
