@@ -1109,6 +1109,7 @@ qf_status ensure_tiled(qf_state* st, ExpPlan* pp) {
     g.chunk0 = (int)wc.size();
     const std::vector<size_t>& idx = kv.second;
     g.nchunk = (int)((idx.size() + qf::kWideTerms - 1) / qf::kWideTerms);
+    g.terms = (int)idx.size();
     for (size_t k = 0; k < idx.size(); k += qf::kWideTerms) {
       qf::WChunk c{};
       qf::WChunkF cf{};
@@ -1944,39 +1945,71 @@ int sparse_run(const RotIn* r, size_t i, size_t nrot, const int32_t* params) {
   return (int)(j - i);
 }
 
-// Fill a TileArgs for rotations [i, j) whose X union fits the tile.
-void build_tile(qf_state* st, const RotIn* r, size_t i, size_t j, uint64_t uni, qf::TileArgs* a) {
+static_assert(qf::kTilePartials <= kPartials, "reverse tile passes' partials");
+
+// The tile of a fused pass: its bits, the low bits it always holds, and how many
+// other bits the union of its X masks may take.
+struct TileShape {
+  int s, room;
+  uint64_t low;
+};
+TileShape tile_shape(const qf_state* st, bool adj) {
   const int n = st->n;
-  const int s_target = std::min(n, st->dt == QF_C128 ? 11 : 12);
-  uint64_t S = uni;
-  for (int b = 0; b < n && popc(S) < s_target; ++b) S |= 1ull << b;
+  if (n < qf::kTileSmall) return {n, n, 0ull};  // the whole state
+  const int s = qf::tile_bits(st->dt, n, adj), l = qf::tile_low_bits(st->dt);
+  return {s, s - l, (1ull << l) - 1};
+}
+// How many of the next `most` rotations (from(k), k = 0, 1, ...) one pass takes.
+template <typename From>
+int tile_run(const TileShape& sh, int most, From&& from, uint64_t* uni) {
+  *uni = 0;
+  int k = 0;
+  for (; k < most; ++k) {
+    const uint64_t u = *uni | from(k).x;
+    if (popc(u & ~sh.low) > sh.room) break;
+    *uni = u;
+  }
+  return k;
+}
+
+// Fill a TileArgs for m rotations (from(k)) with X union uni; *scale is the scale the
+// state keeps aside, s2 (optional) receives its square before each rotation.
+template <typename From>
+void build_tile(const qf_state* st, const TileShape& sh, int m, uint64_t uni, From&& from, double* scale, double* s2,
+                qf::TileArgs* a) {
+  const int n = st->n;
+  uint64_t S = uni | sh.low;
+  for (int b = 0; b < n && popc(S) < sh.s; ++b) S |= 1ull << b;
   std::memset(a, 0, sizeof(*a));
   a->s = popc(S);
   int l = 0;
   while (l < n && ((S >> l) & 1)) ++l;
   a->l = l;
   a->nhi = a->s - l;
+  int local[64];
   int k = 0, kh = 0;
   for (int b = 0; b < n; ++b)
     if ((S >> b) & 1) {
+      local[b] = k;
       a->sbits[k++] = b;
       if (b >= l) a->pos[kh++] = b;
     }
   auto compress = [&](uint64_t v) {
     uint32_t o = 0;
-    for (int q = 0; q < a->s; ++q)
-      if ((v >> a->sbits[q]) & 1) o |= 1u << q;
+    for (uint64_t w = v & S; w; w &= w - 1) o |= 1u << local[__builtin_ctzll(w)];
     return o;
   };
-  a->m = (int)(j - i);
-  for (size_t t = i; t < j; ++t) {
-    qf::TileRot& R = a->r[t - i];
-    R.xl = compress(r[t].x);
-    R.zl = compress(r[t].z & S);
-    R.zout = r[t].z & ~S;
-    R.hl = r[t].x ? 31 - __builtin_clz(R.xl) : -1;
-    R.y = popc(r[t].x & r[t].z);
-    rot_coeffs(st->dt, &st->scale, r[t].th, &R.form, &R.A, &R.B);
+  a->m = m;
+  for (int t = 0; t < m; ++t) {
+    const RotIn& r = from(t);
+    qf::TileRot& R = a->r[t];
+    R.xl = compress(r.x);
+    R.zl = compress(r.z);
+    R.zout = r.z & ~S;
+    R.hl = r.x ? 31 - __builtin_clz(R.xl) : -1;
+    R.y = popc(r.x & r.z);
+    if (s2) s2[t] = *scale * *scale;
+    rot_coeffs(st->dt, scale, r.th, &R.form, &R.A, &R.B);
   }
 }
 
@@ -2002,7 +2035,7 @@ qf_status flush_sector(qf_state* st, std::vector<qf::SecBlk>& pend) {
 
 qf_status apply_rotations(qf_state* st, const RotIn* r, size_t nrot) {
   const int n = st->n;
-  const int umax = std::min(n, 8);
+  const TileShape shape = tile_shape(st, false);
   std::vector<qf::SecBlk> pend;  // sector blocks waiting for one sweep launch
   size_t i = 0;
   while (i < nrot) {
@@ -2029,22 +2062,22 @@ qf_status apply_rotations(qf_state* st, const RotIn* r, size_t nrot) {
         continue;
       }
     }
-    // greedy tile fusion over consecutive rotations whose X support union stays small
-    uint64_t uni = r[i].x;
+    // greedy tile fusion over consecutive rotations whose X union fits a tile
     size_t j = i + 1;
-    while (j < nrot && (int)(j - i) < qf::kTileMaxRot && popc(uni | r[j].x) <= umax) {
+    while (j < nrot && (int)(j - i) < qf::kTileMaxRot) {
       // stop before a run that can become a sparse block
       if (j + 1 < nrot && r[j].x != 0 && r[j + 1].x == r[j].x && r[j].x != r[j - 1].x) break;
-      uni |= r[j].x;
       ++j;
     }
-    if (j - i >= 2 && n >= 4) {
+    uint64_t uni = 0;
+    const int m = tile_run(shape, (int)(j - i), [&](int k) -> const RotIn& { return r[i + k]; }, &uni);
+    if (m >= 2 && n >= 4) {
       qf::TileArgs ta;
-      build_tile(st, r, i, j, uni, &ta);
+      build_tile(st, shape, m, uni, [&](int k) -> const RotIn& { return r[i + k]; }, &st->scale, nullptr, &ta);
       QF_CUDA(qf::launch_tile(st->psi, n, st->dt, ta, st->stream));
-      for (size_t k = i; k < j; ++k) st->real = st->real && keeps_real(r[k].x, r[k].z);
+      for (size_t k = i; k < i + m; ++k) st->real = st->real && keeps_real(r[k].x, r[k].z);
       st->sec_a = st->sec_b = -1;
-      i = j;
+      i += m;
     } else {
       qf::RotArgs a = rot_args(st->dt, &st->scale, r[i].x, r[i].z, r[i].th);
       QF_CUDA(qf::launch_rot(st->psi, n, st->dt, a, st->stream));
@@ -2680,11 +2713,27 @@ static qf_status energy_grad_impl(qf_state* st, uint64_t det, const qf_arot* ans
   st->real = true;
   st->sec_a = st->sec_b = -1;
   QF_CUDA(qf::launch_zero_and_set(st->psi, n, st->dt, det, st->stream));
-  for (const Blk& b : blocks) {
+  const TileShape fshape = tile_shape(st, false), rshape = tile_shape(st, true);
+  for (size_t bi = 0; bi < blocks.size(); ++bi) {
+    const Blk& b = blocks[bi];
     if (b.sparse) {
       const bool rm = qf::sparse_m_real(b.fwd);
       QF_CUDA(qf::launch_sparse(st->psi, n, st->dt, b.fwd, st->real && rm, st->stream));
       st->real = st->real && rm;
+      continue;
+    }
+    // consecutive single rotations share tile passes
+    int most = 1;
+    while (most < qf::kTileMaxRot && bi + most < blocks.size() && !blocks[bi + most].sparse) ++most;
+    uint64_t uni = 0;
+    auto rot = [&](int k) -> const RotIn& { return r[b.i + k]; };
+    const int m = tile_run(fshape, most, rot, &uni);
+    if (m >= 2 && n >= 4) {
+      qf::TileArgs ta;
+      build_tile(st, fshape, m, uni, rot, &st->scale, nullptr, &ta);
+      QF_CUDA(qf::launch_tile(st->psi, n, st->dt, ta, st->stream));
+      for (int k = 0; k < m; ++k) st->real = st->real && keeps_real(rot(k).x, rot(k).z);
+      bi += m - 1;
     } else {
       qf::RotArgs a = rot_args(st->dt, &st->scale, r[b.i].x, r[b.i].z, r[b.i].th);
       QF_CUDA(qf::launch_rot(st->psi, n, st->dt, a, st->stream));
@@ -2735,6 +2784,32 @@ static qf_status energy_grad_impl(qf_state* st, uint64_t det, const qf_arot* ans
                                     st->d_counter, st->d_out + bi, nb, st->stream));
       both_real = both_real && rm;
     } else {
+      int most = 1;
+      while (n >= qf::kTileSmall && most < qf::kTileAdjRot && (size_t)most <= bi && !blocks[bi - most].sparse) ++most;
+      uint64_t uni = 0;
+      RotIn back[qf::kTileAdjRot];  // the inverse rotations, last block first
+      for (int k = 0; k < most; ++k) {
+        back[k] = r[blocks[bi - k].i];
+        back[k].th = -back[k].th;
+      }
+      auto rot = [&](int k) -> const RotIn& { return back[k]; };
+      const int m = tile_run(rshape, most, rot, &uni);
+      if (m >= 2) {
+        qf::TileArgs ta;
+        double sq[qf::kTileAdjRot];
+        build_tile(st, rshape, m, uni, rot, &sc, sq, &ta);
+        ta.lam = st->lam;
+        ta.partials = st->d_partials;
+        ta.counter = st->d_counter;
+        ta.out = st->d_out + bi;
+        QF_CUDA(qf::launch_tile(st->psi, n, st->dt, ta, st->stream));
+        for (int k = 0; k < m; ++k) {
+          s2[bi - k] = sq[k];
+          both_real = both_real && keeps_real(rot(k).x, rot(k).z);
+        }
+        bi -= m - 1;
+        continue;
+      }
       qf::RotArgs a = rot_args(st->dt, &sc, r[b.i].x, r[b.i].z, -r[b.i].th);
       QF_CUDA(qf::launch_adj_rot(st->psi, st->lam, n, st->dt, a, st->d_partials, st->d_counter, st->d_out + bi, nb,
                                  st->stream));

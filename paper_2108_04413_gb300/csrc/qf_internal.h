@@ -52,8 +52,27 @@ struct TileArgs {
   int nhi;      // s - l tile bits above the low run
   int pos[kTileMaxHiBits];  // global positions of those bits, ascending
   int sbits[kTileMaxHiBits + 16];  // all s tile bit positions, ascending
+  // Reverse pass (lam != NULL): rotation t's Im <lam|P|psi> before it is applied goes to
+  // out[-t], then both states take the rotation.  partials holds kTilePartials values.
+  void* lam;
+  double* partials;
+  unsigned* counter;
+  double* out;
   TileRot r[kTileMaxRot];
 };
+constexpr int kTilePartials = 4096;
+// Tiles of the fused rotation passes: 2^s amplitudes that always hold the low bits
+// 0..l-1 (128 bytes), so a pass takes any X masks whose union needs at most s - l other
+// bits.  The large tile (complex64 64 KB, complex128 32 KB; 32 KB each of psi and lam in
+// a reverse pass) from 2^8 tiles on, else 2^10 amplitudes, so that the tiles outnumber
+// the SMs.
+constexpr int kTileSmall = 10;
+inline int tile_low_bits(qf_dtype dt) { return dt == QF_C128 ? 3 : 4; }
+inline int tile_bits(qf_dtype dt, int n, bool adj) {
+  const int big = dt == QF_C128 ? 11 : adj ? 12 : 13;
+  return n >= big + 8 ? big : kTileSmall;
+}
+constexpr int kTileAdjRot = 13;  // rotations of a reverse pass (their partials: 13 x 304 CTAs)
 
 struct SparseArgs {
   int u;        // support qubits (the common x mask)
@@ -133,7 +152,7 @@ struct HGroup {
   uint64_t x;
   int chunk0, nchunk;
   int odd;      // some term has an odd number of Y letters (complex D)
-  int pad;
+  int terms;
 };
 struct WChunk {
   uint64_t z[kWideTerms];

@@ -330,6 +330,288 @@ __global__ void __launch_bounds__(256) k_tile(typename Cx<T>::V* __restrict__ ps
   }
 }
 
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() {
+  asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+}
+
+// ---------------------------------------------------------------------------
+// fused rotation passes on tiles of 2^S amplitudes (S >= 10; k_tile below that)
+//
+// A CTA stages a tile by asynchronous copies, applies the pass's rotations in
+// shared memory and writes it back; three CTAs per SM (large tiles) overlap one's
+// copies with the others' rotations.  Thread tid takes the pairs j0 + o_k,
+// (j0 ^ xl) ^ o_k, with o_k constants (TilePairs), so a pair costs one XOR and the
+// rotation's multiply-adds; its sign is the thread's parity times a sign per k.
+// complex128 is bound by the FP64 pipe (four multiply-adds per pair), complex64 by
+// the state's read and write per pass.
+// ADJ: psi and lam tiles side by side; each rotation first adds its overlap into the
+// thread's own slot in shared memory, summed over the CTA once, after its last tile.
+
+// The pairs of a thread for pivot case C (see PassPairs), in groups of U.
+template <int S, int C> struct TilePairs {
+  static constexpr int P = 1 << (S - 9), KB = S - 9, U = P < 4 ? P : 4;
+  static __device__ __forceinline__ unsigned off(int k) {
+    unsigned o = 0;
+#pragma unroll
+    for (int i = 0; i < KB; ++i)
+      if ((k >> i) & 1) o |= 1u << (C == 0 ? 9 + i : 8 + i < 8 + C ? 8 + i : 9 + i);
+    return o;
+  }
+};
+
+// u' = A u + B i^{3+3y+2p} v, v' = A v + B i^{3+y+2p} u for y odd (YODD) and even; neg: p
+// plus the sign y itself gives.  F: the coefficient form.
+template <int F, bool YODD, typename T, typename V>
+__device__ __forceinline__ void rot_pair(V& u, V& v, T A, T B, unsigned neg) {
+  // the partner's image is (v, -u) for odd y, (i v, i u) for even y; signs go on the
+  // coefficient or by the sign bit (a negated double that feeds a bit operation would
+  // cost an FP64 addition)
+  const V u0 = u, v0 = v;
+  if (F == FORM_B1) {
+    u.x = fma(A, u0.x, YODD ? flip(v0.x, neg) : flip(v0.y, neg ^ 1u));
+    u.y = fma(A, u0.y, YODD ? flip(v0.y, neg) : flip(v0.x, neg));
+    v.x = fma(A, v0.x, YODD ? flip(u0.x, neg ^ 1u) : flip(u0.y, neg ^ 1u));
+    v.y = fma(A, v0.y, YODD ? flip(u0.y, neg ^ 1u) : flip(u0.x, neg));
+  } else {
+    const T b = flip(B, neg), c = flip(B, neg ^ 1u);
+    const bool ab = F == FORM_AB;
+    u.x = fma(YODD ? b : c, YODD ? v0.x : v0.y, ab ? A * u0.x : u0.x);
+    u.y = fma(b, YODD ? v0.y : v0.x, ab ? A * u0.y : u0.y);
+    v.x = fma(c, YODD ? u0.x : u0.y, ab ? A * v0.x : v0.x);
+    v.y = fma(YODD ? c : b, YODD ? u0.y : u0.x, ab ? A * v0.y : v0.y);
+  }
+}
+
+// Running sum of products a * b: FP64, or exact FP32 products in a float pair.
+template <typename T> struct DotAcc;
+template <> struct DotAcc<double> {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <> struct DotAcc<float> {
+  float h = 0.f, l = 0.f;
+  __device__ __forceinline__ void add(float a, float b) {
+    const float p = __fmul_rn(a, b);
+    const float e = fmaf(a, b, -p);
+    const float t = __fadd_rn(h, p);
+    const float bp = __fsub_rn(t, h);
+    const float r = __fadd_rn(__fsub_rn(h, __fsub_rn(t, bp)), __fsub_rn(p, bp));
+    l = __fadd_rn(l, __fadd_rn(r, e));
+    h = t;
+  }
+  __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+};
+
+// One rotation with X part xl != 0 on a tile; the thread's overlap when ADJ.
+template <typename T, int S, int C, int F, bool YODD, bool ADJ>
+__device__ __forceinline__ double tile_pairs(unsigned char* psi, unsigned char* lam, unsigned j0, unsigned xl,
+                                             unsigned zl, unsigned neg0, T A, T B) {
+  using V = typename Cx<T>::V;
+  using TP = TilePairs<S, C>;
+  constexpr unsigned sz = sizeof(V);
+  DotAcc<T> even, odd;  // pairs of positive and negative sign
+#pragma unroll 1
+  for (int kb = 0; kb < TP::P; kb += TP::U) {
+    const unsigned oh = TP::off(kb);
+    const unsigned nh = neg0 ^ (unsigned)__popc(zl & oh);
+    const unsigned a = (j0 + oh) * sz, b = ((j0 ^ xl) ^ oh) * sz;
+#pragma unroll
+    for (int k = 0; k < TP::U; ++k) {
+      const unsigned o = TP::off(k);
+      const unsigned neg = nh ^ (unsigned)__popc(zl & o);
+      V* pu = reinterpret_cast<V*>(psi + a + o * sz);
+      V* pv = reinterpret_cast<V*>(psi + (b ^ (o * sz)));
+      V u = *pu, v = *pv;
+      if (ADJ) {
+        V* qu = reinterpret_cast<V*>(lam + a + o * sz);
+        V* qv = reinterpret_cast<V*>(lam + (b ^ (o * sz)));
+        V p = *qu, r = *qv;
+        // even y: Im conj(p) v + Im conj(r) u; odd y: Re conj(r) u - Re conj(p) v
+        V su = u, sv = v;  // psi with the pair's sign
+        su.x = flip(su.x, neg);
+        su.y = flip(su.y, neg);
+        sv.x = flip(sv.x, neg);
+        sv.y = flip(sv.y, neg);
+        if (YODD) {
+          even.add(r.x, su.x);
+          even.add(r.y, su.y);
+          odd.add(-p.x, sv.x);
+          odd.add(-p.y, sv.y);
+        } else {
+          even.add(p.x, sv.y);
+          even.add(-p.y, sv.x);
+          odd.add(r.x, su.y);
+          odd.add(-r.y, su.x);
+        }
+        rot_pair<F, YODD, T, V>(p, r, A, B, neg);
+        *qu = p;
+        *qv = r;
+      }
+      rot_pair<F, YODD, T, V>(u, v, A, B, neg);
+      *pu = u;
+      *pv = v;
+    }
+  }
+  return ADJ ? even.value() + odd.value() : 0.0;
+}
+
+// A diagonal rotation: out = A u + B i^{3+2p} u.
+template <typename T, int S, int F, bool ADJ>
+__device__ __forceinline__ double tile_diag(unsigned char* psi, unsigned char* lam, unsigned zl, unsigned neg0, T A,
+                                            T B) {
+  using V = typename Cx<T>::V;
+  DotAcc<T> acc;
+#pragma unroll 4
+  for (unsigned j = threadIdx.x; j < (1u << S); j += 256u) {
+    const unsigned p = ((unsigned)__popc(zl & j) + neg0) & 1u;
+    V* pu = reinterpret_cast<V*>(psi) + j;
+    const V u = *pu;
+    if (ADJ) {  // Im conj(lam) s psi
+      V* qu = reinterpret_cast<V*>(lam) + j;
+      const V q = *qu;
+      acc.add(q.x, flip(u.y, p));
+      acc.add(-q.y, flip(u.x, p));
+      *qu = comb<F, T, V>(q, qturn(q, (3u + 2u * p) & 3u), A, B);
+    }
+    *pu = comb<F, T, V>(u, qturn(u, (3u + 2u * p) & 3u), A, B);
+  }
+  return ADJ ? acc.value() : 0.0;
+}
+
+// CTAs per SM.  complex128 forward takes small tiles and many CTAs: with the FP64 pipe
+// saturated, two buffers of the same tile (3 CTAs) or one of twice the size gained
+// nothing (28 qubits, 100 rotations: 122.9 ms against 124.4 and 129).
+template <typename T, int S, bool ADJ> __host__ __device__ constexpr int tile_ctas() {
+  return ADJ ? 2 : sizeof(T) == 8 || S == kTileSmall ? 6 : 3;
+}
+template <typename T, int S, bool ADJ>
+__global__ void __launch_bounds__(256, tile_ctas<T, S, ADJ>())
+    k_tile_pass(typename Cx<T>::V* __restrict__ psi, int n, const __grid_constant__ TileArgs a) {
+  using V = typename Cx<T>::V;
+  constexpr int L = sizeof(T) == 8 ? 3 : 4;
+  constexpr unsigned E16 = 16 / sizeof(V), size = 1u << S;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  unsigned char* tp = smem_raw;                    // psi tile
+  unsigned char* tl = smem_raw + sizeof(V) * size; // lam tile
+  double* red = reinterpret_cast<double*>(tl + sizeof(V) * size);  // [rotation][thread]
+  V* lam = reinterpret_cast<V*>(a.lam);
+  __shared__ uint32_t hitab[1 << (S - L)];  // offsets of the tile's runs of 2^L amplitudes, in units of 2^L
+  const unsigned tid = threadIdx.x;
+  for (unsigned h = tid; h < (1u << (S - L)); h += 256u) {
+    uint32_t off = 0;
+#pragma unroll
+    for (int i = L; i < S; ++i) off |= ((h >> (i - L)) & 1u) << (a.sbits[i] - L);
+    hitab[h] = off;
+  }
+  if (ADJ)
+    for (int r = 0; r < a.m; ++r) red[r * 256 + tid] = 0.0;
+  // launched while the pass before it ends (programmatic dependent launch): all above
+  // reads the arguments only; the states come from the passes before
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const uint64_t ntiles = 1ull << (n - S);
+  auto base_of = [&](uint64_t t) {
+#pragma unroll
+    for (int i = 0; i < S; ++i) t = ins0(t, a.sbits[i]);
+    return t;
+  };
+  auto copy_in = [&](uint64_t base, unsigned char* dst) {
+#pragma unroll 8
+    for (unsigned e = tid * E16; e < size; e += 256u * E16) {
+      const uint64_t g = base | ((uint64_t)hitab[e >> L] << L) | (e & ((1u << L) - 1u));
+      cp_async16(dst + e * sizeof(V), psi + g);
+      if (ADJ) cp_async16(tl + e * sizeof(V), lam + g);
+    }
+  };
+  for (uint64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const uint64_t base = base_of(t);
+    __syncthreads();  // hitab; the last tile's writers are done
+    copy_in(base, tp);
+    cp_async_wait_all();
+    __syncthreads();
+    // the next pass may launch once every CTA is at its last tile's rotations
+    if (t + gridDim.x >= ntiles) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    for (int r = 0; r < a.m; ++r) {
+      const TileRot& R = a.r[r];
+      const unsigned xl = R.xl, zl = R.zl;
+      const int hl = R.hl, form = R.form, y = R.y;
+      const T A = (T)R.A, B = (T)R.B;
+      const unsigned pout = par64(R.zout & base);
+      double d = 0.0;
+      if (hl < 0) {
+        d = form == FORM_A1   ? tile_diag<T, S, FORM_A1, ADJ>(tp, tl, zl, pout, A, B)
+            : form == FORM_B1 ? tile_diag<T, S, FORM_B1, ADJ>(tp, tl, zl, pout, A, B)
+                              : tile_diag<T, S, FORM_AB, ADJ>(tp, tl, zl, pout, A, B);
+      } else {
+        const unsigned j0 = (unsigned)ins0(tid, hl);
+        // the sign of pair k = 0: Z parity of j0, and the one y gives (odd y: - for 1 mod 4; even y: - for 0 mod 4)
+        const unsigned zp = ((unsigned)__popc(zl & j0) + pout) & 1u;
+        const unsigned ys = (y & 1) ? ((y & 2) ? 0u : 1u) : ((y & 2) ? 0u : 1u);
+        auto go = [&](auto c) {
+          constexpr int C = decltype(c)::value;
+          auto run = [&](auto f, auto odd) {
+            return tile_pairs<T, S, C, decltype(f)::value, decltype(odd)::value, ADJ>(tp, tl, j0, xl, zl, zp ^ ys, A,
+                                                                                     B);
+          };
+          using A1 = std::integral_constant<int, FORM_A1>;
+          using B1 = std::integral_constant<int, FORM_B1>;
+          using AB = std::integral_constant<int, FORM_AB>;
+          if (y & 1)
+            d = form == FORM_A1 ? run(A1{}, std::true_type{}) : form == FORM_B1 ? run(B1{}, std::true_type{})
+                                                                               : run(AB{}, std::true_type{});
+          else
+            d = form == FORM_A1 ? run(A1{}, std::false_type{}) : form == FORM_B1 ? run(B1{}, std::false_type{})
+                                                                                : run(AB{}, std::false_type{});
+        };
+        switch (hl) {
+          case 9: go(std::integral_constant<int, 1>{}); break;
+          case 10: go(std::integral_constant<int, (S > 10 ? 2 : 1)>{}); break;
+          case 11: go(std::integral_constant<int, (S > 11 ? 3 : 1)>{}); break;
+          case 12: go(std::integral_constant<int, (S > 12 ? 4 : 1)>{}); break;
+          default: go(std::integral_constant<int, 0>{});
+        }
+        // the overlap's sign: i^y's (y mod 4 >= 2) and the Z parity; tile_pairs took zp ^ ys
+        if (ADJ) d = flip(d, ys ^ ((unsigned)y >> 1));
+      }
+      if (ADJ) red[r * 256 + tid] += d;
+      __syncthreads();
+    }
+#pragma unroll 4
+    for (unsigned e = tid * E16; e < size; e += 256u * E16) {
+      const uint64_t g = base | ((uint64_t)hitab[e >> L] << L) | (e & ((1u << L) - 1u));
+      *reinterpret_cast<float4*>(psi + g) = *reinterpret_cast<const float4*>(tp + e * sizeof(V));
+      if (ADJ) *reinterpret_cast<float4*>(lam + g) = *reinterpret_cast<const float4*>(tl + e * sizeof(V));
+    }
+  }
+  if (!ADJ) return;
+  // the CTA's sums (a warp per rotation), then the last CTA's over the CTAs, in order
+  __shared__ bool last;
+  const int lane = tid & 31, warp = tid >> 5;
+  for (int r = warp; r < a.m; r += 8) {
+    double v = 0.0;
+    for (int j = lane; j < 256; j += 32) v += red[r * 256 + j];
+    v = warp_sum(v);
+    if (lane == 0) a.partials[(size_t)r * gridDim.x + blockIdx.x] = v;
+  }
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) last = atomicAdd(a.counter, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int r = warp; r < a.m; r += 8) {
+    double v = 0.0;
+    for (unsigned j = lane; j < gridDim.x; j += 32) v += __ldcg(a.partials + (size_t)r * gridDim.x + j);
+    v = warp_sum(v);
+    if (lane == 0) a.out[-r] = v;
+  }
+  if (tid == 0) *a.counter = 0u;
+}
+
 // ---------------------------------------------------------------------------
 // sparse composite block
 //
@@ -632,14 +914,6 @@ __global__ void __launch_bounds__(256) k_expect_tiled(const typename Cx<T>::V* _
 // in turn with large ones tile by tile was slower (56 ms: spills).
 // complex64 sums stay in FP32 over four pairs, then join a float pair by TwoSum
 // (converted to FP64 once per tile).
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
-}
-
 template <typename T> struct PassAcc {  // FP64 state: one running sum
   double s = 0.0;
   __device__ __forceinline__ void add(double w, double v) { s = fma(w, v, s); }
@@ -934,8 +1208,19 @@ template <typename T> struct WTab;
 template <> struct WTab<double> { using C = WChunk; using V2 = double2; };
 template <> struct WTab<float> { using C = WChunkF; using V2 = float2; };
 
+// A tile is a chain of one partner tile and one descriptor per class and group, so
+// both come early: the next kHpsiStages - 1 classes' partner tiles are in flight as
+// asynchronous copies, and 64 groups' descriptors at a time are staged in shared
+// memory.  A group of one term needs no table: its weight and sign.
+// 17 qubits, 400 terms (complex128): 748 us one class and one group at a time.
+constexpr int kHpsiStages = 4;
+constexpr int kHpsiBatch = 64;
+struct HpsiRec {
+  uint64_t x, z;   // z: the term's, in a group of one
+  int chunk0, nchunk, flags, pad;  // flags: bit 0 a single term, bit 1 odd, bit 2 even
+};
 template <typename T, int E, bool REALST>
-__global__ void __launch_bounds__(256) k_hpsi_tiled(const typename Cx<T>::V* __restrict__ psi,
+__global__ void __launch_bounds__(256, 2) k_hpsi_tiled(const typename Cx<T>::V* __restrict__ psi,
                                                     typename Cx<T>::V* __restrict__ lam, int n,
                                                     const HClass* __restrict__ classes, int nclasses,
                                                     const HGroup* __restrict__ groups,
@@ -944,8 +1229,10 @@ __global__ void __launch_bounds__(256) k_hpsi_tiled(const typename Cx<T>::V* __r
   using V = typename Cx<T>::V;
   constexpr int TB = (E == 1) ? 8 : (E == 2) ? 9 : (E == 4) ? 10 : (E == 8) ? 11 : 12;
   constexpr int KB = TB - 8;  // bits of k
+  constexpr unsigned E16 = 16 / sizeof(V);
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* tile = reinterpret_cast<V*>(smem_raw);
+  __shared__ HpsiRec rec[kHpsiBatch];
+  __shared__ typename WTab<T>::V2 w1[kHpsiBatch];  // weight of a single term
   const unsigned tid = threadIdx.x;
   const uint64_t ntiles = 1ull << (n - TB);
   double acc_e = 0.0, acc_n = 0.0;
@@ -953,20 +1240,66 @@ __global__ void __launch_bounds__(256) k_hpsi_tiled(const typename Cx<T>::V* __r
     double lx[E], ly[E];
 #pragma unroll
     for (int k = 0; k < E; ++k) lx[k] = ly[k] = 0.0;
+    uint64_t xh_next = nclasses > 0 ? __ldg(&classes[0].xh) : 0;  // of the next class to copy
+    auto copy_in = [&](int ci) {
+      if (ci < nclasses) {
+        V* dst = reinterpret_cast<V*>(smem_raw) + ((ci % kHpsiStages) << TB);
+        const V* src = psi + ((t ^ xh_next) << TB);
+#pragma unroll
+        for (unsigned e = tid * E16; e < (1u << TB); e += 256u * E16) cp_async16(dst + e, src + e);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      if (ci + 1 < nclasses) xh_next = __ldg(&classes[ci + 1].xh);
+    };
+    __syncthreads();  // the last tile's readers are done
+    for (int q = 0; q < kHpsiStages - 1; ++q) copy_in(q);
+    int staged = 0;  // groups [staged - kHpsiBatch, staged) are in rec
     for (int ci = 0; ci < nclasses; ++ci) {
       const HClass C = classes[ci];
       const uint64_t pt = t ^ C.xh;
-      __syncthreads();
-#pragma unroll
-      for (int k = 0; k < E; ++k) tile[tid + 256u * k] = psi[(pt << TB) + tid + 256u * k];
-      __syncthreads();
+      const V* tile = reinterpret_cast<const V*>(smem_raw) + ((ci % kHpsiStages) << TB);
+      asm volatile("cp.async.wait_group %0;" ::"n"(kHpsiStages - 2) : "memory");
+      __syncthreads();  // this class's tile is there, and the last class's readers are done
+      copy_in(ci + kHpsiStages - 1);
       T fx[E], fy[E];
 #pragma unroll
       for (int k = 0; k < E; ++k) fx[k] = fy[k] = 0;
       for (int g = C.g0; g < C.g1; ++g) {
-        const HGroup G = groups[g];
+        if (g >= staged) {  // uniform over the CTA
+          __syncthreads();
+          if (tid < kHpsiBatch && g + (int)tid < classes[nclasses - 1].g1) {
+            const HGroup H = groups[g + tid];
+            const typename WTab<T>::C* W = chunks + H.chunk0;
+            rec[tid] = HpsiRec{H.x, W->z[0], H.chunk0, H.nchunk, (H.terms == 1 ? 1 : 0) | (H.odd ? 2 : 4), 0};
+            w1[tid] = W->tab[0];
+          }
+          staged = g + kHpsiBatch;
+          __syncthreads();
+        }
+        const HpsiRec& G = rec[g - (staged - kHpsiBatch)];
         const unsigned xl = (unsigned)(G.x & ((1ull << TB) - 1ull));
         const unsigned xlo = xl & 255u, xhi = xl >> 8;
+        if (G.flags & 1) {  // D = +-w, real (even y) or imaginary (odd y)
+          const typename WTab<T>::V2 w = w1[g - (staged - kHpsiBatch)];
+          const uint64_t z = G.z;
+          const unsigned zk = (unsigned)(z >> 8) & ((1u << KB) - 1u);
+          const unsigned s0 = par64((z >> TB) & pt) ^ ((unsigned)__popc((unsigned)z & 255u & (tid ^ xlo)) & 1u);
+          const T d = flip((G.flags & 2) ? w.y : w.x, s0);
+#pragma unroll
+          for (int k = 0; k < E; ++k) {
+            const unsigned kk = (unsigned)k ^ xhi;
+            const V v = tile[(tid ^ xlo) | (kk << 8)];
+            const T dk = flip(d, (unsigned)__popc(zk & kk));
+            if (REALST || !(G.flags & 2)) {
+              fx[k] = fma(dk, v.x, fx[k]);
+              if (!REALST) fy[k] = fma(dk, v.y, fy[k]);
+            } else {
+              fx[k] = fma(-dk, v.y, fx[k]);
+              fy[k] = fma(dk, v.x, fy[k]);
+            }
+          }
+          continue;
+        }
         T dx[E], dy[E];
         // the first table initialises D (no add of zero), later tables add to it
         for (int c = 0; c < G.nchunk; ++c) {
@@ -1006,7 +1339,7 @@ __global__ void __launch_bounds__(256) k_hpsi_tiled(const typename Cx<T>::V* __r
           fx[k] = fma(dx[k], v.x, fx[k]);
           if (!REALST) {
             fy[k] = fma(dx[k], v.y, fy[k]);
-            if (G.odd) {
+            if (G.flags & 2) {
               fx[k] = fma(-dy[k], v.y, fx[k]);
               fy[k] = fma(dy[k], v.x, fy[k]);
             }
@@ -1502,9 +1835,53 @@ static cudaError_t tile_impl(void* psi, int n, const TileArgs& a, cudaStream_t s
   return cudaGetLastError();
 }
 
+template <typename T, int S, bool ADJ>
+static cudaError_t tile_pass_t(void* psi, int n, const TileArgs& a, cudaStream_t s) {
+  using V = typename Cx<T>::V;
+  constexpr int tiles_held = ADJ ? 2 : 1;
+  const size_t smem = (sizeof(V) << S) * tiles_held + (ADJ ? a.m * 256 * sizeof(double) : 0);
+  constexpr int most = (int)((sizeof(V) << S) * tiles_held + (ADJ ? kTileAdjRot * 256 * sizeof(double) : 0));
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(k_tile_pass<T, S, ADJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (attr != cudaSuccess) return attr;
+  if (ADJ && (a.m < 1 || a.m > kTileAdjRot)) return cudaErrorInvalidValue;
+  const uint64_t tiles = 1ull << (n - S);
+  uint64_t grid = std::min<uint64_t>(tiles, (uint64_t)sm_count() * tile_ctas<T, S, ADJ>());
+  if (ADJ) grid = std::min<uint64_t>(grid, kTilePartials / a.m);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_tile_pass<T, S, ADJ>, static_cast<V*>(psi), n, a);
+}
+
 cudaError_t launch_tile(void* psi, int n, qf_dtype dt, const TileArgs& a, cudaStream_t s) {
-  const int prof_slot_ = prof_pre(QF_K_TILE, s);
-  cudaError_t e = dt == QF_C128 ? tile_impl<double>(psi, n, a, s) : tile_impl<float>(psi, n, a, s);
+  const bool adj = a.lam != nullptr;
+  const int prof_slot_ = prof_pre(adj ? QF_K_ADJ_ROT : QF_K_TILE, s);
+  cudaError_t e = cudaErrorInvalidValue;
+  if (n < kTileSmall) {
+    if (!adj) e = dt == QF_C128 ? tile_impl<double>(psi, n, a, s) : tile_impl<float>(psi, n, a, s);
+  } else if (dt == QF_C128) {
+    e = adj ? (a.s == 11   ? tile_pass_t<double, 11, true>(psi, n, a, s)
+               : a.s == 10 ? tile_pass_t<double, 10, true>(psi, n, a, s)
+                           : e)
+            : (a.s == 11   ? tile_pass_t<double, 11, false>(psi, n, a, s)
+               : a.s == 10 ? tile_pass_t<double, 10, false>(psi, n, a, s)
+                           : e);
+  } else {
+    e = adj ? (a.s == 12   ? tile_pass_t<float, 12, true>(psi, n, a, s)
+               : a.s == 10 ? tile_pass_t<float, 10, true>(psi, n, a, s)
+                           : e)
+            : (a.s == 13   ? tile_pass_t<float, 13, false>(psi, n, a, s)
+               : a.s == 10 ? tile_pass_t<float, 10, false>(psi, n, a, s)
+                           : e);
+  }
   prof_post(prof_slot_, s);
   count_launch();
   return e;
@@ -1685,30 +2062,20 @@ static cudaError_t hpsi_tiled_e(const void* psi, void* lam, int n, bool realst, 
                                 double* out, int nblocks, cudaStream_t s) {
   using V = typename Cx<T>::V;
   using C = typename WTab<T>::C;
-  const size_t smem = sizeof(V) * 256 * E;
+  const size_t smem = sizeof(V) * 256 * E * kHpsiStages;
   const uint64_t ntiles = 1ull << (n - (8 + (E == 1 ? 0 : E == 2 ? 1 : E == 4 ? 2 : E == 8 ? 3 : 4)));
   // persistent grid: exactly the blocks that are resident at once (a partial
   // second wave would leave most SMs idle at the end)
+  const auto k = realst ? k_hpsi_tiled<T, E, true> : k_hpsi_tiled<T, E, false>;
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int per_sm = 1;
-  if (realst)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hpsi_tiled<T, E, true>, 256, smem);
-  else
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hpsi_tiled<T, E, false>, 256, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem);
   if (per_sm < 1) per_sm = 1;
   uint64_t cap = (uint64_t)sm_count() * (uint64_t)per_sm;
   if (cap > (uint64_t)nblocks) cap = (uint64_t)nblocks;
   unsigned g = (unsigned)std::min<uint64_t>(ntiles, cap);
-  if (realst) {
-    cudaFuncSetAttribute(k_hpsi_tiled<T, E, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_hpsi_tiled<T, E, true><<<g, 256, smem, s>>>(static_cast<const V*>(psi), static_cast<V*>(lam), n, classes,
-                                                  nclasses, groups, static_cast<const C*>(chunks), partials,
-                                                  counter, out);
-  } else {
-    cudaFuncSetAttribute(k_hpsi_tiled<T, E, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_hpsi_tiled<T, E, false><<<g, 256, smem, s>>>(static_cast<const V*>(psi), static_cast<V*>(lam), n, classes,
-                                                   nclasses, groups, static_cast<const C*>(chunks), partials,
-                                                   counter, out);
-  }
+  k<<<g, 256, smem, s>>>(static_cast<const V*>(psi), static_cast<V*>(lam), n, classes, nclasses, groups,
+                         static_cast<const C*>(chunks), partials, counter, out);
   return cudaGetLastError();
 }
 
@@ -1717,15 +2084,11 @@ static cudaError_t hpsi_tiled_t(const void* psi, void* lam, int n, int tb, bool 
                                 int nclasses, const HGroup* groups, const void* chunks, double* partials,
                                 unsigned* counter, double* out, int nblocks, cudaStream_t s) {
   switch (tb) {
-    case 8: return hpsi_tiled_e<T, 1>(psi, lam, n, realst, classes, nclasses, groups, chunks, partials, counter, out, nblocks, s);
-    case 9: return hpsi_tiled_e<T, 2>(psi, lam, n, realst, classes, nclasses, groups, chunks, partials, counter, out, nblocks, s);
     case 10: return hpsi_tiled_e<T, 4>(psi, lam, n, realst, classes, nclasses, groups, chunks, partials, counter, out, nblocks, s);
     case 11: return hpsi_tiled_e<T, 8>(psi, lam, n, realst, classes, nclasses, groups, chunks, partials, counter, out, nblocks, s);
-    case 12: return hpsi_tiled_e<T, 16>(psi, lam, n, realst, classes, nclasses, groups, chunks, partials, counter, out, nblocks, s);
     default: return cudaErrorInvalidValue;
   }
 }
-
 cudaError_t launch_hpsi_tiled(const void* psi, void* lam, int n, qf_dtype dt, int tb, bool realst,
                               const HClass* classes, int nclasses, const HGroup* groups, const void* chunks,
                               double* partials, unsigned* counter, double* out, int nblocks, cudaStream_t s) {
