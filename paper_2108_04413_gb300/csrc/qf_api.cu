@@ -212,6 +212,9 @@ struct qf_state {
   // amplitude has them (set by qf_set_basis, kept by sector-preserving blocks);
   // -1 when unknown.
   int sec_a = -1, sec_b = -1;
+  // Where the amplitudes may be nonzero, as far as this handle's calls tell; checked
+  // against the amplitudes before a call relies on it.
+  qf::Support sup{-1, 0, {}};
   qf::SecBlk* d_secblk = nullptr;  // sector block descriptors (forward, then reverse)
   size_t secblk_cap = 0;
   double* d_sec_partial = nullptr;  // reverse-sweep overlaps per block and CTA
@@ -261,7 +264,7 @@ struct qf_state {
   void* h_sout = nullptr;  // page-locked
   size_t h_sout_cap = 0;
   double* d_partials = nullptr;
-  unsigned* d_counter = nullptr;
+  unsigned* d_counter = nullptr;  // and, in the second word, whether psi leaves `sup`
   double* d_out = nullptr;
   size_t out_cap = 0;
   double* h_out = nullptr;
@@ -1972,15 +1975,51 @@ int tile_run(const TileShape& sh, int most, From&& from, uint64_t* uni) {
   return k;
 }
 
+// The tile's bits for X union uni.
+uint64_t tile_set(const TileShape& sh, int n, uint64_t uni) {
+  uint64_t S = uni | sh.low;
+  for (int b = 0; b < n && popc(S) < sh.s; ++b) S |= 1ull << b;
+  return S;
+}
+
+constexpr int kSupMinQubits = 18;
+void sup_set(qf::Support* s, uint64_t det) {
+  s->d = 0;
+  s->off = det;
+}
+// A rotation with X mask x: every amplitude b also reaches b ^ x.
+void sup_add(qf::Support* s, uint64_t x) {
+  if (s->d < 0) return;
+  for (int i = 0; i < s->d; ++i) x = std::min(x, x ^ s->v[i]);  // clears v's highest bit
+  if (x == 0) return;
+  if (s->d == QF_MAX_QUBITS) {
+    s->d = -1;
+    return;
+  }
+  s->v[s->d++] = x;
+}
+// The tiles with outside bits ~S that hold part of the support (false: all of them).
+bool sup_tiles(const qf::Support& s, int n, uint64_t S, qf::TileArgs* a) {
+  a->nsup = -1;
+  if (s.d < 0) return false;
+  qf::Support o{0, 0, {}};
+  for (int i = 0; i < s.d; ++i) sup_add(&o, s.v[i] & ~S);
+  if (o.d >= n - popc(S)) return false;
+  a->nsup = o.d;
+  a->off = s.off & ~S;
+  for (int i = 0; i < o.d; ++i) a->sup[i] = o.v[i];
+  return true;
+}
+
 // Fill a TileArgs for m rotations (from(k)) with X union uni; *scale is the scale the
 // state keeps aside, s2 (optional) receives its square before each rotation.
 template <typename From>
 void build_tile(const qf_state* st, const TileShape& sh, int m, uint64_t uni, From&& from, double* scale, double* s2,
                 qf::TileArgs* a) {
   const int n = st->n;
-  uint64_t S = uni | sh.low;
-  for (int b = 0; b < n && popc(S) < sh.s; ++b) S |= 1ull << b;
+  const uint64_t S = tile_set(sh, n, uni);
   std::memset(a, 0, sizeof(*a));
+  a->nsup = -1;
   a->s = popc(S);
   int l = 0;
   while (l < n && ((S >> l) & 1)) ++l;
@@ -2037,6 +2076,24 @@ qf_status apply_rotations(qf_state* st, const RotIn* r, size_t nrot) {
   const int n = st->n;
   const TileShape shape = tile_shape(st, false);
   std::vector<qf::SecBlk> pend;  // sector blocks waiting for one sweep launch
+  qf::Support& sup = st->sup;
+  if (!qf::launch_check_support || n < kSupMinQubits) sup.d = -1;
+  bool checked = false;
+  // the tiles a pass needs to visit; the first pass that gains checks the amplitudes
+  auto use_support = [&](qf::TileArgs* ta, uint64_t uni) -> qf_status {
+    if (!sup_tiles(sup, n, tile_set(shape, n, uni), ta)) return QF_OK;
+    if (!checked) {
+      if (sup.d > n - 2) {  // too late in the growth to pay for the check
+        sup.d = ta->nsup = -1;
+        return QF_OK;
+      }
+      QF_CUDA(cudaMemsetAsync(st->d_counter + 1, 0, sizeof(unsigned), st->stream));
+      QF_CUDA(qf::launch_check_support(st->psi, n, st->dt, sup, st->d_counter + 1, st->stream));
+      checked = true;
+    }
+    ta->dense = st->d_counter + 1;
+    return QF_OK;
+  };
   size_t i = 0;
   while (i < nrot) {
     const int run = sparse_run(r, i, nrot, nullptr);
@@ -2045,6 +2102,7 @@ qf_status apply_rotations(qf_state* st, const RotIn* r, size_t nrot) {
       qf::SecBlk sb;
       if (build_sparse(r + i, run, n, false, false, &sa) && to_secblk(sa, n, st->sec_a, st->sec_b, false, &sb)) {
         pend.push_back(sb);
+        sup_add(&sup, r[i].x);
         i += run;
         continue;
       }
@@ -2058,6 +2116,7 @@ qf_status apply_rotations(qf_state* st, const RotIn* r, size_t nrot) {
         QF_CUDA(qf::launch_sparse(st->psi, n, st->dt, sa, st->real && rm, st->stream));
         st->real = st->real && rm;
         st->sec_a = st->sec_b = -1;
+        sup_add(&sup, r[i].x);
         i += run;
         continue;
       }
@@ -2071,11 +2130,17 @@ qf_status apply_rotations(qf_state* st, const RotIn* r, size_t nrot) {
     }
     uint64_t uni = 0;
     const int m = tile_run(shape, (int)(j - i), [&](int k) -> const RotIn& { return r[i + k]; }, &uni);
-    if (m >= 2 && n >= 4) {
+    qf::TileArgs few;  // a single rotation takes a tile pass over half the state or less
+    if ((m >= 2 && n >= 4) || (m == 1 && sup_tiles(sup, n, tile_set(shape, n, uni), &few) && few.nsup < n - shape.s)) {
       qf::TileArgs ta;
       build_tile(st, shape, m, uni, [&](int k) -> const RotIn& { return r[i + k]; }, &st->scale, nullptr, &ta);
+      qf_status us = use_support(&ta, uni);
+      if (us != QF_OK) return us;
       QF_CUDA(qf::launch_tile(st->psi, n, st->dt, ta, st->stream));
-      for (size_t k = i; k < i + m; ++k) st->real = st->real && keeps_real(r[k].x, r[k].z);
+      for (size_t k = i; k < i + m; ++k) {
+        st->real = st->real && keeps_real(r[k].x, r[k].z);
+        sup_add(&sup, r[k].x);
+      }
       st->sec_a = st->sec_b = -1;
       i += m;
     } else {
@@ -2083,6 +2148,7 @@ qf_status apply_rotations(qf_state* st, const RotIn* r, size_t nrot) {
       QF_CUDA(qf::launch_rot(st->psi, n, st->dt, a, st->stream));
       st->real = st->real && keeps_real(r[i].x, r[i].z);
       if (r[i].x != 0) st->sec_a = st->sec_b = -1;  // a diagonal rotation keeps every occupation
+      sup_add(&sup, r[i].x);
       ++i;
     }
   }
@@ -2119,7 +2185,7 @@ qf_status qf_state_create(int n, qf_dtype dtype, void* stream, void* dev_buf, si
     st->own_psi = true;
   }
   if (cudaMalloc(&st->d_partials, kPartials * sizeof(double)) != cudaSuccess ||
-      cudaMalloc(&st->d_counter, sizeof(unsigned)) != cudaSuccess) {
+      cudaMalloc(&st->d_counter, 2 * sizeof(unsigned)) != cudaSuccess) {
     cudaGetLastError();
     if (st->own_psi) cudaFree(st->psi);
     cudaFree(st->d_partials);
@@ -2139,6 +2205,7 @@ qf_status qf_state_create(int n, qf_dtype dtype, void* stream, void* dev_buf, si
     qf_state_destroy(st);
     return fail(QF_ECUDA, std::string("state init: ") + cudaGetErrorString(e));
   }
+  sup_set(&st->sup, 0);
   *out = st;
   return QF_OK;
 }
@@ -2180,6 +2247,7 @@ qf_status qf_set_basis(qf_state* st, uint64_t det) {
   st->real = true;
   st->sec_a = popc(det & kEvenMask);
   st->sec_b = popc(det & ~kEvenMask);
+  sup_set(&st->sup, det);
   QF_CUDA(qf::launch_zero_and_set(st->psi, st->n, st->dt, det, st->stream));
   return QF_OK;
 }
@@ -2193,6 +2261,7 @@ qf_status qf_apply_pauli_exp(qf_state* st, uint64_t x, uint64_t z, double theta)
   QF_CUDA(qf::launch_rot(st->psi, st->n, st->dt, a, st->stream));
   st->real = st->real && keeps_real(x, z);
   if (x != 0) st->sec_a = st->sec_b = -1;
+  sup_add(&st->sup, x);
   return QF_OK;
 }
 
@@ -2484,6 +2553,7 @@ static qf_status energy_grad_impl(qf_state* st, uint64_t det, const qf_arot* ans
     sector = sec_good.load();  // a block that lost the sector form this time: general path
   }
   if (sector) {
+    sup_set(&st->sup, det);
     st->scale = 1.0;
     st->real = true;
     st->sec_a = na;
@@ -2714,12 +2784,15 @@ static qf_status energy_grad_impl(qf_state* st, uint64_t det, const qf_arot* ans
   st->sec_a = st->sec_b = -1;
   QF_CUDA(qf::launch_zero_and_set(st->psi, n, st->dt, det, st->stream));
   const TileShape fshape = tile_shape(st, false), rshape = tile_shape(st, true);
+  qf::Support sup{n < kSupMinQubits ? -1 : 0, det, {}};
+  st->sup.d = -1;
   for (size_t bi = 0; bi < blocks.size(); ++bi) {
     const Blk& b = blocks[bi];
     if (b.sparse) {
       const bool rm = qf::sparse_m_real(b.fwd);
       QF_CUDA(qf::launch_sparse(st->psi, n, st->dt, b.fwd, st->real && rm, st->stream));
       st->real = st->real && rm;
+      sup_add(&sup, r[b.i].x);
       continue;
     }
     // consecutive single rotations share tile passes
@@ -2731,13 +2804,18 @@ static qf_status energy_grad_impl(qf_state* st, uint64_t det, const qf_arot* ans
     if (m >= 2 && n >= 4) {
       qf::TileArgs ta;
       build_tile(st, fshape, m, uni, rot, &st->scale, nullptr, &ta);
+      sup_tiles(sup, n, tile_set(fshape, n, uni), &ta);
       QF_CUDA(qf::launch_tile(st->psi, n, st->dt, ta, st->stream));
-      for (int k = 0; k < m; ++k) st->real = st->real && keeps_real(rot(k).x, rot(k).z);
+      for (int k = 0; k < m; ++k) {
+        st->real = st->real && keeps_real(rot(k).x, rot(k).z);
+        sup_add(&sup, rot(k).x);
+      }
       bi += m - 1;
     } else {
       qf::RotArgs a = rot_args(st->dt, &st->scale, r[b.i].x, r[b.i].z, r[b.i].th);
       QF_CUDA(qf::launch_rot(st->psi, n, st->dt, a, st->stream));
       st->real = st->real && keeps_real(r[b.i].x, r[b.i].z);
+      sup_add(&sup, r[b.i].x);
     }
   }
   const double s_fwd = st->scale;
@@ -3122,6 +3200,7 @@ qf_status multi_small(qf_state* st, uint64_t det, const qf_arot* ansatz, size_t 
   st->real = true;
   st->sec_a = na;
   st->sec_b = nbeta;
+  sup_set(&st->sup, det);
   QF_CUDA(qf::launch_zero_and_set(st->psi, n, st->dt, det, st->stream));
   QF_CUDA(d2h(st->h_sout, st->d_sout, outn * sizeof(double), st->stream));
   QF_CUDA(cudaStreamSynchronize(st->stream));
@@ -3226,6 +3305,7 @@ qf_status qf_state_copy_from_host(qf_state* st, const void* host, size_t bytes) 
   st->scale = 1.0;
   st->real = false;
   st->sec_a = st->sec_b = -1;
+  st->sup.d = -1;
   return QF_OK;
 }
 

@@ -513,8 +513,14 @@ __global__ void __launch_bounds__(256, tile_ctas<T, S, ADJ>())
   // launched while the pass before it ends (programmatic dependent launch): all above
   // reads the arguments only; the states come from the passes before
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const uint64_t ntiles = 1ull << (n - S);
+  const bool part = a.nsup >= 0 && (!a.dense || __ldcg(a.dense) == 0u);
+  const uint64_t ntiles = 1ull << (part ? a.nsup : n - S);
   auto base_of = [&](uint64_t t) {
+    if (part) {
+      uint64_t b = a.off;
+      for (int i = 0; i < a.nsup; ++i) b ^= a.sup[i] & (0ull - ((t >> i) & 1ull));
+      return b;
+    }
 #pragma unroll
     for (int i = 0; i < S; ++i) t = ins0(t, a.sbits[i]);
     return t;
@@ -610,6 +616,30 @@ __global__ void __launch_bounds__(256, tile_ctas<T, S, ADJ>())
     if (lane == 0) a.out[-r] = v;
   }
   if (tid == 0) *a.counter = 0u;
+}
+
+// Whether a state is zero outside a support (one read of the state, half a dense pass):
+// a handle's amplitudes may sit in memory that its owner also writes.
+struct SupportArg {
+  int d;
+  uint64_t off, v[QF_MAX_QUBITS];
+  int top[QF_MAX_QUBITS];
+};
+template <typename V>
+__global__ void __launch_bounds__(256) k_check_support(const V* __restrict__ psi, uint64_t N,
+                                                       const __grid_constant__ SupportArg s, unsigned* dense) {
+  bool out = false;
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+#pragma unroll 8
+  for (uint64_t b = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; b < N; b += stride) {
+    const V a = psi[b];
+    if (a.x == 0 && a.y == 0) continue;
+    uint64_t w = b ^ s.off;
+    for (int i = 0; i < s.d; ++i)
+      if ((w >> s.top[i]) & 1) w ^= s.v[i];
+    out = out || w != 0;
+  }
+  if (out) *dense = 1u;
 }
 
 // ---------------------------------------------------------------------------
@@ -1885,6 +1915,26 @@ cudaError_t launch_tile(void* psi, int n, qf_dtype dt, const TileArgs& a, cudaSt
   prof_post(prof_slot_, s);
   count_launch();
   return e;
+}
+
+cudaError_t launch_check_support(const void* psi, int n, qf_dtype dt, const Support& s, unsigned* dense,
+                                 cudaStream_t stream) {
+  SupportArg a;
+  memset(&a, 0, sizeof(a));
+  a.d = s.d;
+  a.off = s.off;
+  for (int i = 0; i < s.d; ++i) {
+    a.v[i] = s.v[i];
+    a.top[i] = 63 - __builtin_clzll(s.v[i]);
+  }
+  const uint64_t N = 1ull << n;
+  const unsigned g = grid_for(N, 8);
+  if (dt == QF_C128)
+    k_check_support<<<g, 256, 0, stream>>>(static_cast<const double2*>(psi), N, a, dense);
+  else
+    k_check_support<<<g, 256, 0, stream>>>(static_cast<const float2*>(psi), N, a, dense);
+  count_launch();
+  return cudaGetLastError();
 }
 
 template <int NR>
