@@ -1998,16 +1998,23 @@ void sup_add(qf::Support* s, uint64_t x) {
   }
   s->v[s->d++] = x;
 }
-// The tiles with outside bits ~S that hold part of the support (false: all of them).
-bool sup_tiles(const qf::Support& s, int n, uint64_t S, qf::TileArgs* a) {
-  a->nsup = -1;
+// The outside patterns (bits not in S) of the support; false: all of them.  The basis is
+// reduced and ascending, so that neighbouring patterns are near one another in memory.
+bool sup_outside(const qf::Support& s, int n, uint64_t S, qf::Reached* on) {
+  on->nsup = -1;
+  on->dense = nullptr;
   if (s.d < 0) return false;
   qf::Support o{0, 0, {}};
   for (int i = 0; i < s.d; ++i) sup_add(&o, s.v[i] & ~S);
   if (o.d >= n - popc(S)) return false;
-  a->nsup = o.d;
-  a->off = s.off & ~S;
-  for (int i = 0; i < o.d; ++i) a->sup[i] = o.v[i];
+  on->nsup = o.d;
+  on->off = s.off & ~S;
+  std::sort(o.v, o.v + o.d);
+  for (int i = 0; i < o.d; ++i) {
+    uint64_t v = o.v[i];
+    for (int j = i; j-- > 0;) v = std::min(v, v ^ on->sup[j]);
+    on->sup[i] = v;
+  }
   return true;
 }
 
@@ -2019,7 +2026,7 @@ void build_tile(const qf_state* st, const TileShape& sh, int m, uint64_t uni, Fr
   const int n = st->n;
   const uint64_t S = tile_set(sh, n, uni);
   std::memset(a, 0, sizeof(*a));
-  a->nsup = -1;
+  a->on.nsup = -1;
   a->s = popc(S);
   int l = 0;
   while (l < n && ((S >> l) & 1)) ++l;
@@ -2079,19 +2086,19 @@ qf_status apply_rotations(qf_state* st, const RotIn* r, size_t nrot) {
   qf::Support& sup = st->sup;
   if (!qf::launch_check_support || n < kSupMinQubits) sup.d = -1;
   bool checked = false;
-  // the tiles a pass needs to visit; the first pass that gains checks the amplitudes
-  auto use_support = [&](qf::TileArgs* ta, uint64_t uni) -> qf_status {
-    if (!sup_tiles(sup, n, tile_set(shape, n, uni), ta)) return QF_OK;
+  // what a pass over the bits S needs to visit; the first pass that gains checks the amplitudes
+  auto use_support = [&](uint64_t S, qf::Reached* on) -> qf_status {
+    if (!sup_outside(sup, n, S, on)) return QF_OK;
     if (!checked) {
       if (sup.d > n - 2) {  // too late in the growth to pay for the check
-        sup.d = ta->nsup = -1;
+        sup.d = on->nsup = -1;
         return QF_OK;
       }
       QF_CUDA(cudaMemsetAsync(st->d_counter + 1, 0, sizeof(unsigned), st->stream));
       QF_CUDA(qf::launch_check_support(st->psi, n, st->dt, sup, st->d_counter + 1, st->stream));
       checked = true;
     }
-    ta->dense = st->d_counter + 1;
+    on->dense = st->d_counter + 1;
     return QF_OK;
   };
   size_t i = 0;
@@ -2113,7 +2120,13 @@ qf_status apply_rotations(qf_state* st, const RotIn* r, size_t nrot) {
       qf::SparseArgs sa;
       if (build_sparse(r + i, run, n, false, false, &sa)) {
         const bool rm = qf::sparse_m_real(sa);
-        QF_CUDA(qf::launch_sparse(st->psi, n, st->dt, sa, st->real && rm, st->stream));
+        qf::Reached on;
+        qf_status us = use_support(r[i].x, &on);
+        if (us != QF_OK) return us;
+        if (on.nsup >= 0)
+          QF_CUDA(qf::launch_sparse_on(st->psi, n, st->dt, sa, on, st->real && rm, st->stream));
+        else
+          QF_CUDA(qf::launch_sparse(st->psi, n, st->dt, sa, st->real && rm, st->stream));
         st->real = st->real && rm;
         st->sec_a = st->sec_b = -1;
         sup_add(&sup, r[i].x);
@@ -2130,11 +2143,11 @@ qf_status apply_rotations(qf_state* st, const RotIn* r, size_t nrot) {
     }
     uint64_t uni = 0;
     const int m = tile_run(shape, (int)(j - i), [&](int k) -> const RotIn& { return r[i + k]; }, &uni);
-    qf::TileArgs few;  // a single rotation takes a tile pass over half the state or less
-    if ((m >= 2 && n >= 4) || (m == 1 && sup_tiles(sup, n, tile_set(shape, n, uni), &few) && few.nsup < n - shape.s)) {
+    qf::Reached few;  // a single rotation takes a tile pass over half the state or less
+    if ((m >= 2 && n >= 4) || (m == 1 && sup_outside(sup, n, tile_set(shape, n, uni), &few) && few.nsup < n - shape.s)) {
       qf::TileArgs ta;
       build_tile(st, shape, m, uni, [&](int k) -> const RotIn& { return r[i + k]; }, &st->scale, nullptr, &ta);
-      qf_status us = use_support(&ta, uni);
+      qf_status us = use_support(tile_set(shape, n, uni), &ta.on);
       if (us != QF_OK) return us;
       QF_CUDA(qf::launch_tile(st->psi, n, st->dt, ta, st->stream));
       for (size_t k = i; k < i + m; ++k) {
@@ -2804,7 +2817,7 @@ static qf_status energy_grad_impl(qf_state* st, uint64_t det, const qf_arot* ans
     if (m >= 2 && n >= 4) {
       qf::TileArgs ta;
       build_tile(st, fshape, m, uni, rot, &st->scale, nullptr, &ta);
-      sup_tiles(sup, n, tile_set(fshape, n, uni), &ta);
+      sup_outside(sup, n, tile_set(fshape, n, uni), &ta.on);
       QF_CUDA(qf::launch_tile(st->psi, n, st->dt, ta, st->stream));
       for (int k = 0; k < m; ++k) {
         st->real = st->real && keeps_real(rot(k).x, rot(k).z);

@@ -45,6 +45,13 @@ struct TileRot {
   double A, B;
 };
 
+// The values of the bits outside a pass's set that its nonzero amplitudes may have:
+// off ^ (any sum of sup[0..nsup-1]), unless *dense (may be NULL) is nonzero.  nsup = -1: all.
+struct Reached {
+  int nsup;
+  uint64_t off, sup[QF_MAX_QUBITS];
+  const unsigned* dense;
+};
 struct TileArgs {
   int m;        // rotations in this pass
   int s;        // tile bits (2^s amplitudes per tile)
@@ -58,11 +65,7 @@ struct TileArgs {
   double* partials;
   unsigned* counter;
   double* out;
-  // nsup >= 0: every nonzero amplitude lies in a tile with base off ^ (a sum of the sup's),
-  // the only ones the pass visits, unless *dense (may be NULL) is nonzero.
-  int nsup;
-  uint64_t off, sup[QF_MAX_QUBITS];
-  const unsigned* dense;
+  Reached on;
   TileRot r[kTileMaxRot];
 };
 // The indices off ^ (any sum of v[0..d-1]): where a state may be nonzero.  The v's have
@@ -368,6 +371,9 @@ cudaError_t launch_tile(void* psi, int n, qf_dtype dt, const TileArgs& a, cudaSt
 cudaError_t launch_sparse(void* psi, int n, qf_dtype dt, const SparseArgs& a, bool realst, cudaStream_t s);
 bool sparse_m_real(const SparseArgs& a);
 bool sparse_q_imag(const SparseArgs& a);
+// launch_sparse on the outside patterns of `on` (weak: see launch_check_support).
+__attribute__((weak)) cudaError_t launch_sparse_on(void* psi, int n, qf_dtype dt, const SparseArgs& a,
+                                                   const Reached& on, bool realst, cudaStream_t s);
 // *dense = 1 when an amplitude outside s is nonzero (dense zeroed on the stream before).
 // Weak: a build of the planner without the kernels visits every tile.
 __attribute__((weak)) cudaError_t launch_check_support(const void* psi, int n, qf_dtype dt, const Support& s,

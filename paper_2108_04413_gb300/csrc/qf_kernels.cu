@@ -338,6 +338,16 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
 }
 
+// The outside patterns a pass visits (see Reached), after griddepcontrol.wait.
+__device__ __forceinline__ bool on_part(const Reached& r) {
+  return r.nsup >= 0 && (!r.dense || __ldcg(r.dense) == 0u);
+}
+__device__ __forceinline__ uint64_t reached(const Reached& r, uint64_t t) {
+  uint64_t b = r.off;
+  for (int i = 0; i < r.nsup; ++i) b ^= r.sup[i] & (0ull - ((t >> i) & 1ull));
+  return b;
+}
+
 // ---------------------------------------------------------------------------
 // fused rotation passes on tiles of 2^S amplitudes (S >= 10; k_tile below that)
 //
@@ -513,14 +523,10 @@ __global__ void __launch_bounds__(256, tile_ctas<T, S, ADJ>())
   // launched while the pass before it ends (programmatic dependent launch): all above
   // reads the arguments only; the states come from the passes before
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const bool part = a.nsup >= 0 && (!a.dense || __ldcg(a.dense) == 0u);
-  const uint64_t ntiles = 1ull << (part ? a.nsup : n - S);
+  const bool part = on_part(a.on);
+  const uint64_t ntiles = 1ull << (part ? a.on.nsup : n - S);
   auto base_of = [&](uint64_t t) {
-    if (part) {
-      uint64_t b = a.off;
-      for (int i = 0; i < a.nsup; ++i) b ^= a.sup[i] & (0ull - ((t >> i) & 1ull));
-      return b;
-    }
+    if (part) return reached(a.on, t);
 #pragma unroll
     for (int i = 0; i < S; ++i) t = ins0(t, a.sbits[i]);
     return t;
@@ -651,7 +657,7 @@ __global__ void __launch_bounds__(256) k_check_support(const V* __restrict__ psi
 // non-support bits ("outside index").  The arguments hold M - I, so each output
 // is v_r + sum_k (M - I)_rk v_k: the rounding then scales with the (small)
 // change rather than with the amplitude, which keeps complex64 states close to
-// unit norm.  REALM: M is real.  REALST: the state is real (imaginary parts are
+// unit norm.  REALST: the state is real (imaginary parts are
 // exactly zero and stay zero), so only real parts are read and written.
 
 template <int NR>
@@ -677,63 +683,94 @@ __device__ __forceinline__ unsigned sp_class(const SpK<NR>& a, uint64_t base) {
   return cls;
 }
 
-template <typename T, int NR, bool REALM, bool REALST>
-__global__ void __launch_bounds__(256) k_sparse(typename Cx<T>::V* __restrict__ psi, int n,
-                                                const __grid_constant__ SpK<NR> a) {
+// A forward block.  Each of its rotations pairs pattern r with r ^ x, so the composite is
+// a 2x2 matrix per pair of rows: two entries a row, not the block's whole row (a double
+// excitation of equal spins has 6 rows).  For commuting strings of an even number of Y
+// (a Trotter step's) the diagonal is real and the rest imaginary, for an odd number (an
+// excitation's) all is real: FP64 work, which bounds the kernel on large states, is 4
+// multiply-adds a row.  Small ones are bound by the launches, so the next one's
+// prologue overlaps (programmatic dependent launch), and on a state grown from a
+// determinant only the outside patterns it has reached are visited (see Support).
+// Trotter step at 20 qubits, complex128, 2445 blocks: whole rows and every pattern 38 ms,
+// pairs and reached patterns 16 ms.
+enum { PAIR_COMPLEX = 0, PAIR_TURN = 1, PAIR_REAL = 2 };
+template <int NP>
+struct PairK {
+  int u, nzc;
+  int supp[kSparseMaxSupp];
+  uint64_t pat[NP][2], zc[2];
+  Reached on;
+  double2 M[kSparseMaxCls][NP][2][2];  // minus the identity
+};
+
+// out = own + the products of row `own`, in row order.
+template <int F, bool REALST, typename T, typename V>
+__device__ __forceinline__ V pair_row(V own, V first, V second, V m0, V m1, bool own_first) {
+  V o = own;
+  auto mul = [&](V m, V v, bool diag) {
+    if (F == PAIR_COMPLEX || F == PAIR_REAL || diag) {
+      o.x = fma(m.x, v.x, o.x);
+      if (!REALST) o.y = fma(m.x, v.y, o.y);
+    }
+    if (F == PAIR_COMPLEX || (F == PAIR_TURN && !diag)) {
+      o.x = fma(-m.y, v.y, o.x);
+      o.y = fma(m.y, v.x, o.y);
+    }
+  };
+  mul(m0, first, own_first);
+  mul(m1, second, !own_first);
+  return o;
+}
+
+template <typename T, int NP, int F, bool REALST>
+__global__ void __launch_bounds__(256) k_pairs(typename Cx<T>::V* __restrict__ psi, int n,
+                                               const __grid_constant__ PairK<NP> a) {
   using V = typename Cx<T>::V;
-  __shared__ V M[kSparseMaxCls][NR][NR];
-  for (int i = threadIdx.x; i < kSparseMaxCls * NR * NR; i += blockDim.x) {
-    const int c = i / (NR * NR), r = (i / NR) % NR, k = i % NR;
+  __shared__ V M[kSparseMaxCls][NP][2][2];
+  for (int i = threadIdx.x; i < kSparseMaxCls * NP * 4; i += blockDim.x) {
+    const double2 d = (&a.M[0][0][0][0])[i];
     V m;
-    m.x = (T)a.M[c][r][k].x;
-    m.y = (T)a.M[c][r][k].y;
-    M[c][r][k] = m;
+    m.x = (T)d.x;
+    m.y = (T)d.y;
+    (&M[0][0][0][0])[i] = m;
   }
   __syncthreads();
-  const uint64_t nout = 1ull << (n - a.u);
+  // all above reads the arguments only
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const bool part = on_part(a.on);
+  const uint64_t nout = 1ull << (part ? a.on.nsup : n - a.u);
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   T* pr = reinterpret_cast<T*>(psi);
   for (uint64_t o = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; o < nout; o += stride) {
-    const uint64_t base = sp_base(o, a.supp, a.u);
-    const unsigned cls = sp_class(a, base);
-    V v[NR];
+    const uint64_t base = part ? reached(a.on, o) : sp_base(o, a.supp, a.u);
+    unsigned cls = 0;
+    if (a.nzc > 0) cls = par64(a.zc[0] & base);
+    if (a.nzc > 1) cls |= par64(a.zc[1] & base) << 1;
+    V v[NP][2];
 #pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      if (r < a.nr) {
+    for (int p = 0; p < NP; ++p)
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const uint64_t at = base | a.pat[p][r];
         if (REALST) {
-          v[r].x = pr[2 * (base | a.pat[r])];
-          v[r].y = 0;
+          v[p][r].x = pr[2 * at];
+          v[p][r].y = 0;
         } else {
-          v[r] = psi[base | a.pat[r]];
+          v[p][r] = psi[at];
         }
       }
-    }
 #pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      if (r < a.nr) {
-        T ox = v[r].x, oy = v[r].y;
+    for (int p = 0; p < NP; ++p)
 #pragma unroll
-        for (int k = 0; k < NR; ++k) {
-          if (k < a.nr) {
-            const V m = M[cls][r][k];
-            ox = fma(m.x, v[k].x, ox);
-            if (!REALST) oy = fma(m.x, v[k].y, oy);
-            if (!REALM) {
-              ox = fma(-m.y, v[k].y, ox);
-              oy = fma(m.y, v[k].x, oy);
-            }
-          }
-        }
-        if (REALST) {
-          pr[2 * (base | a.pat[r])] = ox;
-        } else {
-          V w;
-          w.x = ox;
-          w.y = oy;
-          psi[base | a.pat[r]] = w;
-        }
+      for (int r = 0; r < 2; ++r) {
+        const V w = pair_row<F, REALST, T, V>(v[p][r], v[p][0], v[p][1], M[cls][p][r][0], M[cls][p][r][1], r == 0);
+        const uint64_t at = base | a.pat[p][r];
+        if (REALST)
+          pr[2 * at] = w.x;
+        else
+          psi[at] = w;
       }
-    }
   }
 }
 
@@ -1974,21 +2011,6 @@ bool sparse_q_imag(const SparseArgs& a) {
 }
 
 template <typename T, int NR>
-static void sparse_fwd(void* psi, int n, const SparseArgs& a, bool realst, cudaStream_t s) {
-  using V = typename Cx<T>::V;
-  const SpK<NR> k = compact<NR>(a);
-  const unsigned g = grid_for(1ull << (n - a.u), 8);
-  V* p = static_cast<V*>(psi);
-  const bool rm = sparse_m_real(a);
-  if (rm && realst)
-    k_sparse<T, NR, true, true><<<g, 256, 0, s>>>(p, n, k);
-  else if (rm)
-    k_sparse<T, NR, true, false><<<g, 256, 0, s>>>(p, n, k);
-  else
-    k_sparse<T, NR, false, false><<<g, 256, 0, s>>>(p, n, k);
-}
-
-template <typename T, int NR>
 static void sparse_adj(void* psi, void* lam, int n, const SparseArgs& a, bool realst, double* partials,
                        unsigned* counter, double* out, int nblocks, cudaStream_t s) {
   using V = typename Cx<T>::V;
@@ -2004,14 +2026,77 @@ static void sparse_adj(void* psi, void* lam, int n, const SparseArgs& a, bool re
     k_adj_sparse<T, NR, false, false><<<nblocks, 256, 0, s>>>(p, l, n, k, partials, counter, out);
 }
 
+template <typename T, int NP, int F>
+static cudaError_t pairs_t(void* psi, int n, const SparseArgs& a, const uint64_t (*pat)[2], const int (*row)[2],
+                           const Reached& on, bool realst, cudaStream_t s) {
+  using V = typename Cx<T>::V;
+  PairK<NP> k;
+  memset(&k, 0, sizeof(k));
+  k.u = a.u;
+  k.nzc = a.nzc;
+  for (int i = 0; i < a.u; ++i) k.supp[i] = a.supp[i];
+  k.zc[0] = a.zc[0];
+  k.zc[1] = a.zc[1];
+  k.on = on;
+  for (int p = 0; p < NP; ++p)
+    for (int r = 0; r < 2; ++r) {
+      k.pat[p][r] = pat[p][r];
+      for (int c = 0; c < a.ncls; ++c)
+        for (int q = 0; q < 2; ++q)
+          if (row[p][r] >= 0 && row[p][q] >= 0) k.M[c][p][r][q] = a.M[c][row[p][r]][row[p][q]];
+    }
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid_for(1ull << (n - a.u), 8));
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  V* v = static_cast<V*>(psi);
+  if (F == PAIR_REAL && realst) return cudaLaunchKernelEx(&cfg, k_pairs<T, NP, PAIR_REAL, true>, v, n, k);
+  return cudaLaunchKernelEx(&cfg, k_pairs<T, NP, F, false>, v, n, k);
+}
+template <typename T, int NP>
+static cudaError_t pairs_f(void* psi, int n, const SparseArgs& a, const uint64_t (*pat)[2], const int (*row)[2],
+                           const Reached& on, int form, bool realst, cudaStream_t s) {
+  return form == PAIR_REAL   ? pairs_t<T, NP, PAIR_REAL>(psi, n, a, pat, row, on, realst, s)
+         : form == PAIR_TURN ? pairs_t<T, NP, PAIR_TURN>(psi, n, a, pat, row, on, false, s)
+                             : pairs_t<T, NP, PAIR_COMPLEX>(psi, n, a, pat, row, on, false, s);
+}
 template <typename T>
-static void sparse_fwd_nr(void* psi, int n, const SparseArgs& a, bool realst, cudaStream_t s) {
-  if (a.nr <= 2)
-    sparse_fwd<T, 2>(psi, n, a, realst, s);
-  else if (a.nr <= 4)
-    sparse_fwd<T, 4>(psi, n, a, realst, s);
-  else
-    sparse_fwd<T, 8>(psi, n, a, realst, s);
+static cudaError_t pairs(void* psi, int n, const SparseArgs& a, const Reached& on, bool realst, cudaStream_t s) {
+  uint64_t x = 0, pat[2 * kSparseMaxRows][2];
+  for (int i = 0; i < a.u; ++i) x |= 1ull << a.supp[i];
+  int row[2 * kSparseMaxRows][2], np = 0;
+  for (int r = 0; r < a.nr; ++r) {  // rows ascend, so a pair's lower row comes first
+    int q = 0;
+    while (q < a.nr && a.pat[q] != (a.pat[r] ^ x)) ++q;
+    if (q < r) continue;
+    const bool alone = q == a.nr, low = a.pat[r] < (a.pat[r] ^ x);
+    pat[np][low ? 0 : 1] = a.pat[r];
+    pat[np][low ? 1 : 0] = a.pat[r] ^ x;
+    row[np][low ? 0 : 1] = r;
+    row[np++][low ? 1 : 0] = alone ? -1 : q;
+  }
+  bool real = true, turn = true;
+  for (int c = 0; c < a.ncls; ++c)
+    for (int r = 0; r < a.nr; ++r)
+      for (int q = 0; q < a.nr; ++q) {
+        real = real && a.M[c][r][q].y == 0.0;
+        turn = turn && (r == q ? a.M[c][r][q].y : a.M[c][r][q].x) == 0.0;
+      }
+  const int form = real ? PAIR_REAL : turn ? PAIR_TURN : PAIR_COMPLEX;
+  cudaError_t e = cudaSuccess;
+  for (int p = 0; p < np && e == cudaSuccess; p += 4) {  // the pairs are independent
+    const int m = std::min(4, np - p);
+    e = m == 1   ? pairs_f<T, 1>(psi, n, a, pat + p, row + p, on, form, realst, s)
+        : m == 2 ? pairs_f<T, 2>(psi, n, a, pat + p, row + p, on, form, realst, s)
+        : m == 3 ? pairs_f<T, 3>(psi, n, a, pat + p, row + p, on, form, realst, s)
+                 : pairs_f<T, 4>(psi, n, a, pat + p, row + p, on, form, realst, s);
+  }
+  return e;
 }
 
 template <typename T>
@@ -2025,15 +2110,21 @@ static void sparse_adj_nr(void* psi, void* lam, int n, const SparseArgs& a, bool
     sparse_adj<T, 8>(psi, lam, n, a, realst, partials, counter, out, nblocks, s);
 }
 
-cudaError_t launch_sparse(void* psi, int n, qf_dtype dt, const SparseArgs& a, bool realst, cudaStream_t s) {
+cudaError_t launch_sparse_on(void* psi, int n, qf_dtype dt, const SparseArgs& a, const Reached& on, bool realst,
+                             cudaStream_t s) {
   const int prof_slot_ = prof_pre(QF_K_SPARSE, s);
-  if (dt == QF_C128)
-    sparse_fwd_nr<double>(psi, n, a, realst, s);
-  else
-    sparse_fwd_nr<float>(psi, n, a, realst, s);
+  const cudaError_t e = dt == QF_C128 ? pairs<double>(psi, n, a, on, realst, s)
+                                      : pairs<float>(psi, n, a, on, realst, s);
   prof_post(prof_slot_, s);
   count_launch();
-  return cudaGetLastError();
+  return e;
+}
+
+cudaError_t launch_sparse(void* psi, int n, qf_dtype dt, const SparseArgs& a, bool realst, cudaStream_t s) {
+  Reached all;
+  memset(&all, 0, sizeof(all));
+  all.nsup = -1;
+  return launch_sparse_on(psi, n, dt, a, all, realst, s);
 }
 
 cudaError_t launch_expect(const void* psi, int n, qf_dtype dt, const ExpGroup* groups, int ngroups,

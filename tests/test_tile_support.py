@@ -84,3 +84,48 @@ def test_amplitudes_written_by_their_owner(dtype, tol, where):
     st.apply_circuit(abi.as_rots(*(list(c) for c in zip(*rots))))
     st.fold_scale()
     assert float((buf.to(torch.complex128) - _reference(n, rots, ref)).abs().max()) < tol
+
+
+@pytest.mark.parametrize("orbitals,electrons,steps", [(4, 3, 2), (5, 5, 1), (9, 7, 2)])
+@pytest.mark.parametrize("dtype,tol", [("c128", 1e-12), ("c64", 2e-5)])
+def test_trotter_blocks(orbitals, electrons, steps, dtype, tol):
+    """Composite blocks of one to three row pairs, real and imaginary links, before and
+    after the state has reached every pattern."""
+    from paper_2108_04413_gb300 import prep
+
+    n = 2 * orbitals
+    rng = np.random.default_rng(orbitals)
+    h = rng.normal(size=(orbitals, orbitals))
+    g = rng.normal(size=(orbitals,) * 4)
+    g = g + g.transpose(1, 0, 2, 3)
+    g = g + g.transpose(0, 1, 3, 2)
+    g = g + g.transpose(2, 3, 0, 1)
+    terms = prep.molecular_hamiltonian(h + h.T, 0.2 * g)
+    xs = np.unique(terms["x"])
+    same = [x for x in xs if bin(int(x)).count("1") == 4 and bin(int(x) & 0x155555).count("1") in (0, 4)]
+    keep = list(rng.choice(xs, size=min(len(xs), 12), replace=False)) + same[:3]
+    terms = terms[np.isin(terms["x"], keep)]
+    kind = torch.complex128 if dtype == "c128" else torch.complex64
+    buf = torch.empty(1 << n, dtype=kind, device="cuda")
+    st = qf.State(n, dtype, buffer=buf)
+    det = (1 << electrons) - 1
+    ansatz, _ = prep.uccsd_ansatz(orbitals, electrons)
+    real = prep.bind_thetas(ansatz, rng.normal(0, 0.3, size=int(ansatz["param"].max()) + 1))[:40]
+    for start in ("determinant", "turned", "written"):
+        st.set_basis(det)
+        ref = torch.zeros(1 << n, dtype=torch.complex128, device="cuda")
+        ref[det] = 1.0
+        if start == "turned":  # excitations' real blocks on a complex state
+            st.apply_pauli_exp(3, 1, 0.4)
+            st.apply_pauli_exp(0, 2, 0.4)
+            ref = _reference(n, [(3, 1, 0.4), (0, 2, 0.4)], ref)
+            st.apply_circuit(real)
+            ref = _reference(n, list(zip(real["x"].tolist(), real["z"].tolist(), real["theta"].tolist())), ref)
+        if start == "written":
+            st.from_numpy(np.full(1 << n, 2.0 ** (-n / 2), dtype=np.complex128 if dtype == "c128" else np.complex64))
+            ref = torch.full_like(ref, 2.0 ** (-n / 2))
+        st.trotter(terms, 0.3, steps)
+        st.fold_scale()
+        for _ in range(steps):
+            ref = _reference(n, [(int(t["x"]), int(t["z"]), float(t["coeff"]) * 0.3 / steps) for t in terms], ref)
+        assert float((buf.to(torch.complex128) - ref).abs().max()) < tol
