@@ -2079,8 +2079,36 @@ qf_status flush_sector(qf_state* st, std::vector<qf::SecBlk>& pend) {
   return check_barrier(st);
 }
 
-qf_status apply_rotations(qf_state* st, const RotIn* r, size_t nrot) {
+// Move to the front of r[0..window) the rotations of one tile pass: those whose X masks
+// fit the tile and that commute with every rotation they overtake.  Returns how many.
+// 27 qubits, 300 random rotations, complex64: 85 passes in list order, 77 gathered
+// (34.1 and 32.4 ms); 28 qubits, 100, complex128: 83.8 and 79.7 ms.  A longer window than
+// 96, or taking the masks that add the fewest bits first, gave no fewer passes.
+constexpr int kTileWindow = 96;
+int tile_gather(const TileShape& sh, RotIn* r, int window, uint64_t* uni) {
+  RotIn later[kTileWindow];
+  *uni = 0;
+  int m = 0, nl = 0, k = 0;
+  for (; k < window && m < qf::kTileMaxRot; ++k) {
+    const RotIn c = r[k];
+    bool take = popc((*uni | c.x) & ~sh.low) <= sh.room;
+    for (int q = 0; take && q < nl; ++q)
+      take = ((popc(c.x & later[q].z) ^ popc(c.z & later[q].x)) & 1) == 0;
+    if (take) {
+      *uni |= c.x;
+      r[m++] = c;
+    } else {
+      later[nl++] = c;
+    }
+  }
+  std::copy(later, later + nl, r + m);
+  return m;
+}
+
+qf_status apply_rotations(qf_state* st, const RotIn* list, size_t nrot) {
   const int n = st->n;
+  std::vector<RotIn> order(list, list + nrot);
+  RotIn* r = order.data();
   const TileShape shape = tile_shape(st, false);
   std::vector<qf::SecBlk> pend;  // sector blocks waiting for one sweep launch
   qf::Support& sup = st->sup;
@@ -2134,15 +2162,15 @@ qf_status apply_rotations(qf_state* st, const RotIn* r, size_t nrot) {
         continue;
       }
     }
-    // greedy tile fusion over consecutive rotations whose X union fits a tile
+    // tile fusion: the rotations of a window that fit one tile
     size_t j = i + 1;
-    while (j < nrot && (int)(j - i) < qf::kTileMaxRot) {
+    while (j < nrot && (int)(j - i) < kTileWindow) {
       // stop before a run that can become a sparse block
       if (j + 1 < nrot && r[j].x != 0 && r[j + 1].x == r[j].x && r[j].x != r[j - 1].x) break;
       ++j;
     }
     uint64_t uni = 0;
-    const int m = tile_run(shape, (int)(j - i), [&](int k) -> const RotIn& { return r[i + k]; }, &uni);
+    const int m = tile_gather(shape, r + i, (int)(j - i), &uni);
     qf::Reached few;  // a single rotation takes a tile pass over half the state or less
     if ((m >= 2 && n >= 4) || (m == 1 && sup_outside(sup, n, tile_set(shape, n, uni), &few) && few.nsup < n - shape.s)) {
       qf::TileArgs ta;
