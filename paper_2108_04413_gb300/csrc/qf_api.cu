@@ -2105,6 +2105,54 @@ int tile_gather(const TileShape& sh, RotIn* r, int window, uint64_t* uni) {
   return m;
 }
 
+// A composite block waiting for a pass over a tile (see k_block_pass).
+struct QueuedBlock {
+  qf::SparseArgs sa;
+  uint64_t x;
+  bool real;  // sparse_m_real
+};
+// Whether a block has the form of a BlockRec; its pairs' rows (lower first).
+bool block_pairs(const qf::SparseArgs& a, uint64_t x, bool real, int (*row)[2]) {
+  if (a.nzc > 1 || (a.nr & 1) || a.nr > 2 * qf::kPassPairs) return false;
+  int np = 0;
+  for (int r = 0; r < a.nr; ++r) {
+    int q = 0;
+    while (q < a.nr && a.pat[q] != (a.pat[r] ^ x)) ++q;
+    if (q == a.nr) return false;
+    if (q > r) row[np][0] = r, row[np++][1] = q;
+  }
+  if (real) return true;
+  for (int c = 0; c < a.ncls; ++c)
+    for (int r = 0; r < a.nr; ++r)
+      for (int q = 0; q < a.nr; ++q)
+        if ((r == q ? a.M[c][r][q].y : a.M[c][r][q].x) != 0.0) return false;
+  return true;
+}
+void fill_block(const qf::SparseArgs& a, uint64_t x, uint64_t S, const int* local, bool real, qf::BlockRec* R) {
+  int row[qf::kSparseMaxRows][2];
+  block_pairs(a, x, real, row);
+  auto compress = [&](uint64_t v) {
+    uint32_t o = 0;
+    for (uint64_t w = v & S; w; w &= w - 1) o |= 1u << local[__builtin_ctzll(w)];
+    return o;
+  };
+  R->u = a.u;
+  R->np = a.nr / 2;
+  R->turn = !real;
+  for (int i = 0; i < a.u; ++i) R->supp[i] = (uint8_t)local[a.supp[i]];
+  R->zl = a.nzc ? compress(a.zc[0]) : 0;
+  R->zout = a.nzc ? a.zc[0] & ~S : 0;
+  for (int p = 0; p < R->np; ++p) {
+    R->pat[p][0] = (uint16_t)compress(a.pat[row[p][0]]);
+    R->pat[p][1] = (uint16_t)compress(a.pat[row[p][1]]);
+    for (int c = 0; c < a.ncls; ++c)
+      for (int i = 0; i < 4; ++i) {
+        const double2 m = a.M[c][row[p][i >> 1]][row[p][i & 1]];
+        R->M[c][p][i] = real || i == 0 || i == 3 ? m.x : m.y;
+      }
+  }
+}
+
 qf_status apply_rotations(qf_state* st, const RotIn* list, size_t nrot) {
   const int n = st->n;
   std::vector<RotIn> order(list, list + nrot);
@@ -2129,10 +2177,51 @@ qf_status apply_rotations(qf_state* st, const RotIn* list, size_t nrot) {
     on->dense = st->d_counter + 1;
     return QF_OK;
   };
+  // Blocks of one pass (three or more: a pass moves the whole state once, a block alone
+  // its active rows, a quarter or less, by a launch of its own).
+  std::vector<QueuedBlock> queue;  // queue[nq]: the block being built
+  int nq = 0;
+  uint64_t quni = 0;
+  const int bs = n >= qf::kTileSmall && qf::launch_block_pass ? qf::block_tile_bits(st->dt, n) : 0;
+  const TileShape bshape{bs, bs - qf::tile_low_bits(st->dt), (1ull << qf::tile_low_bits(st->dt)) - 1};
+  auto flush_blocks = [&]() -> qf_status {
+    if (nq >= 3) {
+      const uint64_t S = tile_set(bshape, n, quni);
+      qf::BlockPass bp;
+      std::memset(&bp, 0, sizeof(bp));
+      bp.s = bs;
+      bp.nb = nq;
+      int local[64], k = 0;
+      for (int b = 0; b < n; ++b)
+        if ((S >> b) & 1) local[b] = k, bp.sbits[k++] = b;
+      for (int q = 0; q < nq; ++q) fill_block(queue[q].sa, queue[q].x, S, local, queue[q].real, &bp.b[q]);
+      qf_status us = use_support(S, &bp.on);
+      if (us != QF_OK) return us;
+      QF_CUDA(qf::launch_block_pass(st->psi, n, st->dt, bp, st->stream));
+    }
+    for (int q = 0; q < nq; ++q) {
+      const QueuedBlock& b = queue[q];
+      if (nq < 3) {
+        qf::Reached on;
+        qf_status us = use_support(b.x, &on);
+        if (us != QF_OK) return us;
+        if (on.nsup >= 0)
+          QF_CUDA(qf::launch_sparse_on(st->psi, n, st->dt, b.sa, on, st->real && b.real, st->stream));
+        else
+          QF_CUDA(qf::launch_sparse(st->psi, n, st->dt, b.sa, st->real && b.real, st->stream));
+      }
+      st->real = st->real && b.real;
+      sup_add(&sup, b.x);
+    }
+    if (nq) st->sec_a = st->sec_b = -1;
+    nq = 0;
+    quni = 0;
+    return QF_OK;
+  };
   size_t i = 0;
   while (i < nrot) {
     const int run = sparse_run(r, i, nrot, nullptr);
-    if (run >= 2 && st->sec_a >= 0 && st->real) {
+    if (nq == 0 && run >= 2 && st->sec_a >= 0 && st->real) {
       qf::SparseArgs sa;
       qf::SecBlk sb;
       if (build_sparse(r + i, run, n, false, false, &sa) && to_secblk(sa, n, st->sec_a, st->sec_b, false, &sb)) {
@@ -2145,23 +2234,32 @@ qf_status apply_rotations(qf_state* st, const RotIn* list, size_t nrot) {
     qf_status fs = flush_sector(st, pend);
     if (fs != QF_OK) return fs;
     if (run >= 2) {
-      qf::SparseArgs sa;
+      if (queue.empty()) queue.resize(qf::kPassBlocks + 1);
+      qf::SparseArgs& sa = queue[nq].sa;
       if (build_sparse(r + i, run, n, false, false, &sa)) {
+        const uint64_t x = r[i].x;
         const bool rm = qf::sparse_m_real(sa);
-        qf::Reached on;
-        qf_status us = use_support(r[i].x, &on);
-        if (us != QF_OK) return us;
-        if (on.nsup >= 0)
-          QF_CUDA(qf::launch_sparse_on(st->psi, n, st->dt, sa, on, st->real && rm, st->stream));
-        else
-          QF_CUDA(qf::launch_sparse(st->psi, n, st->dt, sa, st->real && rm, st->stream));
-        st->real = st->real && rm;
-        st->sec_a = st->sec_b = -1;
-        sup_add(&sup, r[i].x);
+        int row[qf::kSparseMaxRows][2];
+        const bool fits = bs && popc(x & ~bshape.low) <= bshape.room && block_pairs(sa, x, rm, row);
+        if (nq && (!fits || nq == qf::kPassBlocks || popc((quni | x) & ~bshape.low) > bshape.room)) {
+          const int at = nq;
+          qf_status us = flush_blocks();
+          if (us != QF_OK) return us;
+          queue[0].sa = queue[at].sa;
+        }
+        queue[nq].x = x;
+        queue[nq++].real = rm;
+        quni |= x;
+        if (!fits) {
+          qf_status us = flush_blocks();
+          if (us != QF_OK) return us;
+        }
         i += run;
         continue;
       }
     }
+    qf_status bf = flush_blocks();
+    if (bf != QF_OK) return bf;
     // tile fusion: the rotations of a window that fit one tile
     size_t j = i + 1;
     while (j < nrot && (int)(j - i) < kTileWindow) {
@@ -2193,6 +2291,8 @@ qf_status apply_rotations(qf_state* st, const RotIn* list, size_t nrot) {
       ++i;
     }
   }
+  qf_status bf = flush_blocks();
+  if (bf != QF_OK) return bf;
   return flush_sector(st, pend);
 }
 

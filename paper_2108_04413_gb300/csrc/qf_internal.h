@@ -89,6 +89,30 @@ inline int tile_bits(qf_dtype dt, int n, bool adj) {
   const int big = dt == QF_C128 ? 11 : adj ? 12 : 13;
   return n >= big + 8 ? big : kTileSmall;
 }
+// A pass of consecutive composite blocks on one tile: for each, the 2x2 matrices of its
+// row pairs (see k_block_pass).
+constexpr int kPassBlocks = 24, kPassPairs = 3;
+struct BlockRec {
+  uint8_t supp[kSparseMaxSupp];  // support bits, tile-local, ascending
+  int u, np;
+  int turn;                      // links imaginary (diagonal real); else all real
+  uint32_t zl;                   // the outside Z mask within the tile
+  uint64_t zout;                 // and outside it
+  uint16_t pat[kPassPairs][2];   // the pairs' rows, tile-local
+  double M[2][kPassPairs][4];    // per class and pair: minus the identity, row by row
+};
+struct BlockPass {
+  int s, nb;
+  int sbits[kTileMaxHiBits + 16];
+  Reached on;
+  BlockRec b[kPassBlocks];
+};
+// The tile of a block pass: a step costs a barrier more than it costs arithmetic, so the
+// large tile already from 2^5 tiles on.
+inline int block_tile_bits(qf_dtype dt, int n) {
+  const int big = dt == QF_C128 ? 11 : 13;
+  return n >= big + 5 ? big : kTileSmall;
+}
 constexpr int kTileAdjRot = 13;  // rotations of a reverse pass (their partials: 13 x 304 CTAs)
 
 struct SparseArgs {
@@ -374,6 +398,9 @@ bool sparse_q_imag(const SparseArgs& a);
 // launch_sparse on the outside patterns of `on` (weak: see launch_check_support).
 __attribute__((weak)) cudaError_t launch_sparse_on(void* psi, int n, qf_dtype dt, const SparseArgs& a,
                                                    const Reached& on, bool realst, cudaStream_t s);
+// Weak: see launch_check_support.
+__attribute__((weak)) cudaError_t launch_block_pass(void* psi, int n, qf_dtype dt, const BlockPass& a,
+                                                    cudaStream_t s);
 // *dense = 1 when an amplitude outside s is nonzero (dense zeroed on the stream before).
 // Weak: a build of the planner without the kernels visits every tile.
 __attribute__((weak)) cudaError_t launch_check_support(const void* psi, int n, qf_dtype dt, const Support& s,

@@ -774,6 +774,90 @@ __global__ void __launch_bounds__(256) k_pairs(typename Cx<T>::V* __restrict__ p
   }
 }
 
+// Consecutive forward blocks on tiles of 2^S amplitudes in shared memory (see k_tile_pass
+// and k_pairs): one launch, and one read and write of the state, for up to kPassBlocks
+// blocks, with a CTA barrier between them.  A thread takes one pair of rows at one
+// outside pattern of the tile.  Trotter step at 20 qubits, complex128, 2445 blocks: 16 ms one
+// launch each, 5.9 ms in 300 launches (20 us a pass: barriers, and the FP64 pipe where all
+// tiles are reached).
+template <typename T, int S>
+__global__ void __launch_bounds__(256, (sizeof(typename Cx<T>::V) << S) > 32768 ? 3 : 4)
+    k_block_pass(typename Cx<T>::V* __restrict__ psi, int n, const __grid_constant__ BlockPass a) {
+  using V = typename Cx<T>::V;
+  constexpr int L = sizeof(T) == 8 ? 3 : 4;
+  constexpr unsigned E16 = 16 / sizeof(V), size = 1u << S;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  V* tile = reinterpret_cast<V*>(smem_raw);
+  __shared__ uint32_t hitab[1 << (S - L)];
+  __shared__ T M[kPassBlocks][2][kPassPairs][4];
+  const unsigned tid = threadIdx.x;
+  for (unsigned h = tid; h < (1u << (S - L)); h += 256u) {
+    uint32_t off = 0;
+#pragma unroll
+    for (int i = L; i < S; ++i) off |= ((h >> (i - L)) & 1u) << (a.sbits[i] - L);
+    hitab[h] = off;
+  }
+  for (int i = tid; i < a.nb * 8 * kPassPairs; i += 256)
+    (&M[0][0][0][0])[i] = (T)(&a.b[i / (8 * kPassPairs)].M[0][0][0])[i % (8 * kPassPairs)];
+  // all above reads the arguments only
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const bool part = on_part(a.on);
+  const uint64_t ntiles = 1ull << (part ? a.on.nsup : n - S);
+  for (uint64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    uint64_t base = t;
+    if (part) {
+      base = reached(a.on, t);
+    } else {
+#pragma unroll
+      for (int i = 0; i < S; ++i) base = ins0(base, a.sbits[i]);
+    }
+    __syncthreads();  // hitab and M; the last tile's writers are done
+#pragma unroll 8
+    for (unsigned e = tid * E16; e < size; e += 256u * E16)
+      cp_async16(tile + e, psi + (base | ((uint64_t)hitab[e >> L] << L) | (e & ((1u << L) - 1u))));
+    cp_async_wait_all();
+    __syncthreads();
+    if (t + gridDim.x >= ntiles) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    for (int b = 0; b < a.nb; ++b) {
+      const BlockRec& R = a.b[b];
+      const int ob = S - R.u;
+      const unsigned items = (unsigned)R.np << ob;
+      const unsigned pout = par64(R.zout & base), zl = R.zl;
+      for (unsigned i = tid; i < items; i += 256u) {
+        const unsigned p = i >> ob;
+        unsigned j = i & ((1u << ob) - 1u);
+        for (int q = 0; q < R.u; ++q) {
+          const unsigned low = j & ((1u << R.supp[q]) - 1u);
+          j = ((j - low) << 1) | low;
+        }
+        const T* m = M[b][((unsigned)__popc(zl & j) + pout) & 1u][p];
+        V* pu = tile + (j | R.pat[p][0]);
+        V* pv = tile + (j | R.pat[p][1]);
+        const V u = *pu, v = *pv;
+        V x = u, y = v;
+        if (R.turn) {
+          x.x = fma(-m[1], v.y, fma(m[0], u.x, x.x));
+          x.y = fma(m[1], v.x, fma(m[0], u.y, x.y));
+          y.x = fma(m[3], v.x, fma(-m[2], u.y, y.x));
+          y.y = fma(m[3], v.y, fma(m[2], u.x, y.y));
+        } else {
+          x.x = fma(m[1], v.x, fma(m[0], u.x, x.x));
+          x.y = fma(m[1], v.y, fma(m[0], u.y, x.y));
+          y.x = fma(m[3], v.x, fma(m[2], u.x, y.x));
+          y.y = fma(m[3], v.y, fma(m[2], u.y, y.y));
+        }
+        *pu = x;
+        *pv = y;
+      }
+      __syncthreads();
+    }
+#pragma unroll 4
+    for (unsigned e = tid * E16; e < size; e += 256u * E16)
+      *reinterpret_cast<float4*>(psi + (base | ((uint64_t)hitab[e >> L] << L) | (e & ((1u << L) - 1u)))) =
+          *reinterpret_cast<const float4*>(tile + e);
+  }
+}
+
 // ---------------------------------------------------------------------------
 // expectation value, pair form
 //
@@ -1972,6 +2056,37 @@ cudaError_t launch_check_support(const void* psi, int n, qf_dtype dt, const Supp
     k_check_support<<<g, 256, 0, stream>>>(static_cast<const float2*>(psi), N, a, dense);
   count_launch();
   return cudaGetLastError();
+}
+
+template <typename T, int S>
+static cudaError_t block_pass_t(void* psi, int n, const BlockPass& a, cudaStream_t s) {
+  using V = typename Cx<T>::V;
+  constexpr size_t smem = sizeof(V) << S;
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(k_block_pass<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (attr != cudaSuccess) return attr;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)std::min<uint64_t>(1ull << (n - S), (uint64_t)sm_count() * (smem > 32768 ? 3 : 4)));
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_block_pass<T, S>, static_cast<V*>(psi), n, a);
+}
+
+cudaError_t launch_block_pass(void* psi, int n, qf_dtype dt, const BlockPass& a, cudaStream_t s) {
+  const int prof_slot_ = prof_pre(QF_K_SPARSE, s);
+  const cudaError_t e = dt == QF_C128 ? (a.s == 11 ? block_pass_t<double, 11>(psi, n, a, s)
+                                                   : block_pass_t<double, kTileSmall>(psi, n, a, s))
+                                      : (a.s == 13 ? block_pass_t<float, 13>(psi, n, a, s)
+                                                   : block_pass_t<float, kTileSmall>(psi, n, a, s));
+  prof_post(prof_slot_, s);
+  count_launch();
+  return e;
 }
 
 template <int NR>

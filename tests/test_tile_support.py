@@ -86,9 +86,10 @@ def test_amplitudes_written_by_their_owner(dtype, tol, where):
     assert float((buf.to(torch.complex128) - _reference(n, rots, ref)).abs().max()) < tol
 
 
-@pytest.mark.parametrize("orbitals,electrons,steps", [(4, 3, 2), (5, 5, 1), (9, 7, 2)])
+@pytest.mark.parametrize("orbitals,electrons,steps,count", [(4, 3, 2, 12), (5, 5, 1, 12), (5, 4, 1, 999),
+                                                            (7, 6, 1, 999), (9, 7, 2, 12), (9, 8, 1, 150)])
 @pytest.mark.parametrize("dtype,tol", [("c128", 1e-12), ("c64", 2e-5)])
-def test_trotter_blocks(orbitals, electrons, steps, dtype, tol):
+def test_trotter_blocks(orbitals, electrons, steps, count, dtype, tol):
     """Composite blocks of one to three row pairs, real and imaginary links, before and
     after the state has reached every pattern."""
     from paper_2108_04413_gb300 import prep
@@ -103,7 +104,8 @@ def test_trotter_blocks(orbitals, electrons, steps, dtype, tol):
     terms = prep.molecular_hamiltonian(h + h.T, 0.2 * g)
     xs = np.unique(terms["x"])
     same = [x for x in xs if bin(int(x)).count("1") == 4 and bin(int(x) & 0x155555).count("1") in (0, 4)]
-    keep = list(rng.choice(xs, size=min(len(xs), 12), replace=False)) + same[:3]
+    few = rng.choice(xs, size=min(len(xs), 12), replace=False)
+    keep = list(few if count == 12 else xs[:count]) + same[:3]
     terms = terms[np.isin(terms["x"], keep)]
     kind = torch.complex128 if dtype == "c128" else torch.complex64
     buf = torch.empty(1 << n, dtype=kind, device="cuda")
