@@ -2163,8 +2163,8 @@ qf_status apply_rotations(qf_state* st, const RotIn* list, size_t nrot) {
   if (!qf::launch_check_support || n < kSupMinQubits) sup.d = -1;
   bool checked = false;
   // what a pass over the bits S needs to visit; the first pass that gains checks the amplitudes
-  auto use_support = [&](uint64_t S, qf::Reached* on) -> qf_status {
-    if (!sup_outside(sup, n, S, on)) return QF_OK;
+  auto use_span = [&](const qf::Support& span, uint64_t S, qf::Reached* on) -> qf_status {
+    if (!sup_outside(span, n, S, on)) return QF_OK;
     if (!checked) {
       if (sup.d > n - 2) {  // too late in the growth to pay for the check
         sup.d = on->nsup = -1;
@@ -2177,6 +2177,7 @@ qf_status apply_rotations(qf_state* st, const RotIn* list, size_t nrot) {
     on->dense = st->d_counter + 1;
     return QF_OK;
   };
+  auto use_support = [&](uint64_t S, qf::Reached* on) { return use_span(sup, S, on); };
   // Blocks of one pass (three or more: a pass moves the whole state once, a block alone
   // its active rows, a quarter or less, by a launch of its own).
   std::vector<QueuedBlock> queue;  // queue[nq]: the block being built
@@ -2260,6 +2261,40 @@ qf_status apply_rotations(qf_state* st, const RotIn* list, size_t nrot) {
     }
     qf_status bf = flush_blocks();
     if (bf != QF_OK) return bf;
+    // A long run of one X mask; below kPhaseMin strings a sine and cosine a pair cost more
+    // FP64 operations (about 60 and one a string) than the rotations (four a string).
+    // complex64 stays on the tiles: its rotations run at the FP32 rate.
+    int len = run;
+    if (r[i].x == 0)
+      while (i + len < nrot && r[i + len].x == 0) ++len;
+    if (len >= qf::kPhaseMin && st->dt == QF_C128 && qf::launch_phase_run) {
+      len = std::min(len, qf::kPhaseMax);
+      qf::PhaseArgs pa;
+      pa.m = len;
+      pa.x = r[i].x;
+      pa.h = hibit(pa.x);
+      pa.y = popc(pa.x & r[i].z) & 3;
+      for (int k = 0; k < len; ++k) {
+        pa.z[k] = r[i + k].z;
+        pa.th[k] = ((popc(pa.x & r[i + k].z) - pa.y) & 2) ? -r[i + k].th : r[i + k].th;
+      }
+      // b: the reached indices with bit h cleared by x
+      qf::Support span = sup;
+      sup_add(&span, pa.x);
+      if (pa.x) {
+        for (int k = 0; k < span.d; ++k)
+          if ((span.v[k] >> pa.h) & 1) span.v[k] ^= pa.x;
+        if ((span.off >> pa.h) & 1) span.off ^= pa.x;
+      }
+      qf_status us = use_span(span, pa.x ? 1ull << pa.h : 0, &pa.on);
+      if (us != QF_OK) return us;
+      QF_CUDA(qf::launch_phase_run(st->psi, n, pa, st->stream));
+      st->real = st->real && keeps_real(r[i].x, r[i].z);
+      if (pa.x != 0) st->sec_a = st->sec_b = -1;
+      sup_add(&sup, pa.x);
+      i += len;
+      continue;
+    }
     // tile fusion: the rotations of a window that fit one tile
     size_t j = i + 1;
     while (j < nrot && (int)(j - i) < kTileWindow) {

@@ -107,6 +107,19 @@ struct BlockPass {
   Reached on;
   BlockRec b[kPassBlocks];
 };
+// A run of commuting rotations with one X mask: the rotation of a pair (b, b ^ x) by the
+// signed sum of their angles (see k_phase_run).
+constexpr int kPhaseMax = 256, kPhaseMin = 24;
+struct PhaseArgs {
+  int m;
+  int h;       // highest set bit of x, -1 when x == 0
+  int y;       // popc(x & z) mod 4 of the first; the others' signs against it are in th
+  int pad;
+  uint64_t x;
+  Reached on;  // values of b, the pair's index with bit h clear
+  uint64_t z[kPhaseMax];
+  double th[kPhaseMax];
+};
 // The tile of a block pass: a step costs a barrier more than it costs arithmetic, so the
 // large tile already from 2^5 tiles on.
 inline int block_tile_bits(qf_dtype dt, int n) {
@@ -401,6 +414,8 @@ __attribute__((weak)) cudaError_t launch_sparse_on(void* psi, int n, qf_dtype dt
 // Weak: see launch_check_support.
 __attribute__((weak)) cudaError_t launch_block_pass(void* psi, int n, qf_dtype dt, const BlockPass& a,
                                                     cudaStream_t s);
+// complex128 only.  Weak: see launch_check_support.
+__attribute__((weak)) cudaError_t launch_phase_run(void* psi, int n, const PhaseArgs& a, cudaStream_t s);
 // *dense = 1 when an amplitude outside s is nonzero (dense zeroed on the stream before).
 // Weak: a build of the planner without the kernels visits every tile.
 __attribute__((weak)) cudaError_t launch_check_support(const void* psi, int n, qf_dtype dt, const Support& s,

@@ -774,6 +774,50 @@ __global__ void __launch_bounds__(256) k_pairs(typename Cx<T>::V* __restrict__ p
   }
 }
 
+// A run of commuting rotations of one X mask, too varied in Z for a composite (a Trotter
+// step's one-electron flips, each with a Z on every other qubit; its diagonal): on the pair
+// (b, b ^ x) their product is one rotation by phi(b), the sum of the angles with signs
+// (-1)^{popc(z & b)}.  Bound by the FP64 pipe: one addition a string and one sine and cosine
+// a pair, where a rotation each takes four multiply-adds a string and pair.
+// Trotter step at 20 qubits, 3631 strings in 91 runs: 7.8 ms as tile passes, 1.4 ms.
+__global__ void __launch_bounds__(256) k_phase_run(double2* __restrict__ psi, int n,
+                                                   const __grid_constant__ PhaseArgs a) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const bool part = on_part(a.on);
+  const uint64_t nout = 1ull << (part ? a.on.nsup : a.h < 0 ? n : n - 1);
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t o = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; o < nout; o += stride) {
+    const uint64_t b = part ? reached(a.on, o) : a.h < 0 ? o : ins0(o, a.h);
+    double phi = 0.0;
+#pragma unroll 4
+    for (int k = 0; k < a.m; ++k) phi += flip(a.th[k], par64(a.z[k] & b));
+    double sn, cs;
+    sincos(phi, &sn, &cs);
+    const double2 u = psi[b];
+    if (a.h < 0) {
+      double2 w;
+      w.x = fma(sn, u.y, cs * u.x);
+      w.y = fma(-sn, u.x, cs * u.y);
+      psi[b] = w;
+      continue;
+    }
+    const double2 v = psi[b ^ a.x];
+    // v' = cos v - i i^y sin u, u' = cos u - i conj(i^y) sin v
+    const double s = (a.y & 2) ? -sn : sn;
+    double2 p, q;
+    if (a.y & 1) {
+      p = make_double2(fma(-s, v.x, cs * u.x), fma(-s, v.y, cs * u.y));
+      q = make_double2(fma(s, u.x, cs * v.x), fma(s, u.y, cs * v.y));
+    } else {
+      p = make_double2(fma(s, v.y, cs * u.x), fma(-s, v.x, cs * u.y));
+      q = make_double2(fma(s, u.y, cs * v.x), fma(-s, u.x, cs * v.y));
+    }
+    psi[b] = p;
+    psi[b ^ a.x] = q;
+  }
+}
+
 // Consecutive forward blocks on tiles of 2^S amplitudes in shared memory (see k_tile_pass
 // and k_pairs): one launch, and one read and write of the state, for up to kPassBlocks
 // blocks, with a CTA barrier between them.  A thread takes one pair of rows at one
@@ -2056,6 +2100,23 @@ cudaError_t launch_check_support(const void* psi, int n, qf_dtype dt, const Supp
     k_check_support<<<g, 256, 0, stream>>>(static_cast<const float2*>(psi), N, a, dense);
   count_launch();
   return cudaGetLastError();
+}
+
+cudaError_t launch_phase_run(void* psi, int n, const PhaseArgs& a, cudaStream_t s) {
+  const int prof_slot_ = prof_pre(QF_K_TILE, s);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid_for(1ull << (a.h < 0 ? n : n - 1), 8));
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_phase_run, static_cast<double2*>(psi), n, a);
+  prof_post(prof_slot_, s);
+  count_launch();
+  return e;
 }
 
 template <typename T, int S>

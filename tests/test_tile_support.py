@@ -131,3 +131,34 @@ def test_trotter_blocks(orbitals, electrons, steps, count, dtype, tol):
         for _ in range(steps):
             ref = _reference(n, [(int(t["x"]), int(t["z"]), float(t["coeff"]) * 0.3 / steps) for t in terms], ref)
         assert float((buf.to(torch.complex128) - ref).abs().max()) < tol
+
+
+@pytest.mark.parametrize("n,count", [(1, 30), (6, 24), (13, 40), (18, 300), (19, 23)])
+@pytest.mark.parametrize("parity", [0, 1])
+@pytest.mark.parametrize("dtype,tol", [("c128", 1e-12), ("c64", 2e-5)])
+def test_runs_of_one_x_mask(n, count, parity, dtype, tol):
+    """Commuting strings of one X mask, all with an even or all with an odd number of Y, and
+    a diagonal run, on a determinant, on a spread state and on one written by its owner."""
+    rng = np.random.default_rng([n, count, parity])
+    kind = torch.complex128 if dtype == "c128" else torch.complex64
+    buf = torch.empty(1 << n, dtype=kind, device="cuda")
+    st = qf.State(n, dtype, buffer=buf)
+    det = (1 << n) // 3
+    st.set_basis(det)
+    ref = torch.zeros(1 << n, dtype=torch.complex128, device="cuda")
+    ref[det] = 1.0
+    for step in range(4):
+        x = int(rng.integers(1, 1 << n)) if step != 2 else 0
+        rots = []
+        while len(rots) < count:
+            z = int(rng.integers(0, 1 << n))
+            if x == 0 or bin(x & z).count("1") % 2 == parity:
+                rots.append((x, z, float(rng.uniform(-math.pi, math.pi))))
+        if step == 3:
+            st.fold_scale()
+            buf.copy_(torch.full_like(buf, 2.0 ** (-n / 2)))
+            ref = buf.to(torch.complex128, copy=True)
+        st.apply_circuit(abi.as_rots(*(list(c) for c in zip(*rots))))
+        ref = _reference(n, rots, ref)
+    st.fold_scale()
+    assert float((buf.to(torch.complex128) - ref).abs().max()) < tol
