@@ -2111,6 +2111,76 @@ struct QueuedBlock {
   uint64_t x;
   bool real;  // sparse_m_real
 };
+// Which indices within each tile (bits S) of a block pass are reached, from the span
+// before it and its blocks' X masks, all of which lie in S: every tile holds a shifted
+// copy of the span's part in S.  A block needs the outside patterns that go with a row of
+// its pairs (of a molecular Trotter step, a quarter: both spins' parities are fixed).
+void fill_reached(const qf::Support& sup, int n, uint64_t S, const int* local, const std::vector<QueuedBlock>& q,
+                  qf::BlockPass* bp) {
+  auto compress = [&](uint64_t v) {
+    uint32_t o = 0;
+    for (uint64_t w = v & S; w; w &= w - 1) o |= 1u << local[__builtin_ctzll(w)];
+    return o;
+  };
+  qf::Support in{0, 0, {}};
+  for (int b = 0; b < bp->nb; ++b) sup_add(&in, q[b].x);
+  // on.sup is the reduced basis of the span outside S; a span vector's part outside S is a
+  // sum of those whose highest bits it has
+  uint64_t lift[QF_MAX_QUBITS];
+  bool have[QF_MAX_QUBITS] = {};
+  std::vector<std::pair<uint64_t, uint64_t>> key;  // (sum of on.sup's as a bit set, vector in S)
+  for (int i = 0; i < sup.d; ++i) {
+    uint64_t set = 0;
+    for (int j = 0; j < bp->on.nsup; ++j)
+      if ((sup.v[i] >> hibit(bp->on.sup[j])) & 1) set |= 1ull << j;
+    key.emplace_back(set, sup.v[i] & S);
+  }
+  // Gauss-Jordan on the bit sets: one vector for each single on.sup, the rest lie in S
+  for (int j = 0; j < bp->on.nsup; ++j) {
+    size_t at = 0;
+    while (at < key.size() && (!((key[at].first >> j) & 1) || [&] {
+      for (int m = 0; m < j; ++m)
+        if (have[m] && lift[m] == at) return true;
+      return false;
+    }())) ++at;
+    if (at == key.size()) return;  // not the projection of this span (bp->b[].nin stay at "all")
+    have[j] = true;
+    lift[j] = at;
+    for (size_t m = 0; m < key.size(); ++m)
+      if (m != at && ((key[m].first >> j) & 1)) key[m].first ^= key[at].first, key[m].second ^= key[at].second;
+  }
+  for (size_t m = 0; m < key.size(); ++m)
+    if (key[m].first == 0) sup_add(&in, key[m].second);
+  for (int j = 0; j < bp->on.nsup; ++j) bp->lsup[j] = (uint16_t)compress(key[lift[j]].second);
+  bp->loff = (uint16_t)compress(sup.off);
+  for (int b = 0; b < bp->nb; ++b) {
+    const uint64_t x = q[b].x;
+    qf::Support rest{0, 0, {}}, key{0, 0, {}};  // outside the support; on it, x aside
+    uint64_t lift[qf::kSparseMaxSupp];
+    for (int i = 0; i < in.d; ++i) {
+      uint64_t w = in.v[i];
+      if ((w >> hibit(x)) & 1) w ^= x;
+      for (int l = 0; l < key.d; ++l)
+        if ((w >> hibit(key.v[l])) & 1) w ^= lift[l];
+      if (w & x) {
+        lift[key.d] = w;
+        key.v[key.d++] = w & x;
+      } else {
+        sup_add(&rest, w);
+      }
+    }
+    qf::Reached w;
+    if (!sup_outside(rest, n, (((1ull << n) - 1) & ~S) | x, &w)) continue;
+    qf::BlockRec& R = bp->b[b];
+    R.nin = w.nsup;
+    R.supp_mask = compress(x);
+    R.omask = compress(~x);
+    R.nlift = key.d;
+    for (int l = 0; l < key.d; ++l) R.lift[l] = (uint16_t)compress(lift[l]);
+    for (int i = 0; i < w.nsup; ++i) R.in[i] = (uint16_t)compress(w.sup[i]);
+  }
+}
+
 // Whether a block has the form of a BlockRec; its pairs' rows (lower first).
 bool block_pairs(const qf::SparseArgs& a, uint64_t x, bool real, int (*row)[2]) {
   if (a.nzc > 1 || (a.nr & 1) || a.nr > 2 * qf::kPassPairs) return false;
@@ -2138,6 +2208,7 @@ void fill_block(const qf::SparseArgs& a, uint64_t x, uint64_t S, const int* loca
   };
   R->u = a.u;
   R->np = a.nr / 2;
+  R->nin = popc(S);  // every pattern
   R->turn = !real;
   for (int i = 0; i < a.u; ++i) R->supp[i] = (uint8_t)local[a.supp[i]];
   R->zl = a.nzc ? compress(a.zc[0]) : 0;
@@ -2198,6 +2269,7 @@ qf_status apply_rotations(qf_state* st, const RotIn* list, size_t nrot) {
       for (int q = 0; q < nq; ++q) fill_block(queue[q].sa, queue[q].x, S, local, queue[q].real, &bp.b[q]);
       qf_status us = use_support(S, &bp.on);
       if (us != QF_OK) return us;
+      if (bp.on.nsup >= 0) fill_reached(sup, n, S, local, queue, &bp);
       QF_CUDA(qf::launch_block_pass(st->psi, n, st->dt, bp, st->stream));
     }
     for (int q = 0; q < nq; ++q) {

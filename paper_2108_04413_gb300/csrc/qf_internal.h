@@ -99,12 +99,21 @@ struct BlockRec {
   uint32_t zl;                   // the outside Z mask within the tile
   uint64_t zout;                 // and outside it
   uint16_t pat[kPassPairs][2];   // the pairs' rows, tile-local
+  // The outside patterns of a tile at which a pair is reached: the tile's reached index
+  // (see BlockPass), moved by the lifts to the pair's lower row on the support (never, if
+  // they cannot), then ^ (any sum of in[0..nin-1]).  nin >= s - u: every pattern.
+  int nin, nlift;
+  uint32_t supp_mask, omask;     // the support (x) and the tile's other bits
+  uint16_t lift[kSparseMaxSupp];  // with distinct highest support bits
+  uint16_t in[kTileMaxHiBits + 16];
   double M[2][kPassPairs][4];    // per class and pair: minus the identity, row by row
 };
 struct BlockPass {
   int s, nb;
   int sbits[kTileMaxHiBits + 16];
   Reached on;
+  // a reached index within tile on.off ^ (sum of on.sup's): loff ^ (sum of the same lsup's)
+  uint16_t loff, lsup[QF_MAX_QUBITS];
   BlockRec b[kPassBlocks];
 };
 // A run of commuting rotations with one X mask: the rotation of a pair (b, b ^ x) by the

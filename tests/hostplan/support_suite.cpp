@@ -1,8 +1,8 @@
 // Circuits on a determinant, planned by the C ABI and carried out on the host exactly as
 // launched: each pass touches only the tiles, outside patterns or pairs it is told to visit.
 //   support_suite <n> <det> <c128|c64> <rots.bin> [<det written by the owner in between>]
-// prints the status, the largest deviation from the rotations applied one by one, and how
-// many launches visited a part of the state.  The launchers replaced here are those that
+// prints the status, the largest deviation from the rotations applied one by one, how many
+// launches visited a part of the state and how many blocks a part of their tiles.  The launchers replaced here are those that
 // cuda_stub.cpp, compiled with them renamed, would only record.
 #include <cmath>
 #include <complex>
@@ -15,7 +15,7 @@
 #include "qf_internal.h"
 
 typedef std::complex<double> cplx;
-static int parts = 0;
+static int parts = 0, inner = 0;
 static int par(uint64_t v) { return __builtin_parityll(v); }
 static const cplx kI[4] = {{1, 0}, {0, 1}, {-1, 0}, {0, -1}};
 
@@ -114,15 +114,43 @@ cudaError_t launch_sparse(void* p, int n, qf_dtype dt, const SparseArgs& a, bool
 }
 cudaError_t launch_block_pass(void* p, int n, qf_dtype dt, const BlockPass& a, cudaStream_t) {
   const Amp psi{p, dt};
-  for (uint64_t base : visited(a.on, n, expand(~0ull, a.sbits, a.s)))
+  const bool part = a.on.nsup >= 0 && (!a.on.dense || *a.on.dense == 0);
+  uint64_t t = 0;
+  for (uint64_t base : visited(a.on, n, expand(~0ull, a.sbits, a.s))) {
+    uint64_t in_tile = a.loff;
+    for (int i = 0; part && i < a.on.nsup; ++i)
+      if ((t >> i) & 1) in_tile ^= a.lsup[i];
+    ++t;
     for (int b = 0; b < a.nb; ++b) {
       const BlockRec& R = a.b[b];
       uint64_t supp = 0;
       for (int i = 0; i < R.u; ++i) supp |= 1ull << R.supp[i];
-      for (uint64_t j = 0; j < (1ull << a.s); ++j) {
-        if (j & supp) continue;
-        const int c = par(R.zl & j) ^ par(R.zout & base);
-        for (int q = 0; q < R.np; ++q) {
+      const bool some = part && R.nin < a.s - R.u;
+      inner += some;
+      auto patterns = [&](int q) {  // of pair q
+        std::vector<uint64_t> js;
+        if (!some) {
+          for (uint64_t j = 0; j < (1ull << a.s); ++j)
+            if (!(j & supp)) js.push_back(j);
+          return js;
+        }
+        if (R.supp_mask != supp || R.omask != ((1ull << a.s) - 1 & ~supp)) std::abort();
+        uint64_t w = in_tile;
+        if (w >> R.supp[R.u - 1] & 1) w ^= supp;
+        for (int l = 0; l < R.nlift; ++l)
+          if ((w ^ R.pat[q][0]) >> (63 - __builtin_clzll(R.lift[l] & supp)) & 1) w ^= R.lift[l];
+        if ((w ^ R.pat[q][0]) & supp) return js;
+        for (uint64_t o = 0; o < (1ull << R.nin); ++o) {
+          uint64_t j = w & R.omask;
+          for (int i = 0; i < R.nin; ++i)
+            if ((o >> i) & 1) j ^= R.in[i];
+          js.push_back(j);
+        }
+        return js;
+      };
+      for (int q = 0; q < R.np; ++q)
+        for (uint64_t j : patterns(q)) {
+          const int c = par(R.zl & j) ^ par(R.zout & base);
           const double* m = R.M[c][q];
           const cplx l = R.turn ? cplx(0, 1) : cplx(1, 0);
           const uint64_t iu = base | expand(j | R.pat[q][0], a.sbits, a.s), iv = base | expand(j | R.pat[q][1], a.sbits, a.s);
@@ -130,8 +158,8 @@ cudaError_t launch_block_pass(void* p, int n, qf_dtype dt, const BlockPass& a, c
           psi.set(iu, u + m[0] * u + l * m[1] * v);
           psi.set(iv, v + l * m[2] * u + m[3] * v);
         }
-      }
     }
+  }
   return cudaSuccess;
 }
 cudaError_t launch_phase_run(void* p, int n, const PhaseArgs& a, cudaStream_t) {
@@ -185,7 +213,7 @@ int main(int argc, char** argv) {
   double scale = 1, worst = 0;
   qf_state_info(st, nullptr, nullptr, nullptr, &scale);
   for (uint64_t b = 0; b < N; ++b) worst = std::max(worst, std::abs(scale * Amp{p, dt}.get(b) - ref[b]));
-  std::printf("%d %.3g %d\n", (int)s, worst, parts);
+  std::printf("%d %.3g %d %d\n", (int)s, worst, parts, inner);
   qf_state_destroy(st);
   return 0;
 }

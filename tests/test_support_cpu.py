@@ -35,7 +35,7 @@ def _run(suite, path, n, rots, dtype, written=()):
     abi.as_rots(*(list(c) for c in zip(*rots))).tofile(path / "rots.bin")
     out = subprocess.run([suite, str(n), str((1 << n) // 3), dtype, str(path / "rots.bin"), *map(str, written)],
                          check=True, capture_output=True, text=True, timeout=600).stdout.split()
-    return int(out[0]), float(out[1]), int(out[2])
+    return int(out[0]), float(out[1]), int(out[2]), int(out[3])
 
 
 def _random(n, count, rng):
@@ -51,7 +51,7 @@ def _random(n, count, rng):
 @pytest.mark.parametrize("dtype,tol", [("c128", 1e-12), ("c64", 2e-5)])
 @pytest.mark.parametrize("n,count", [(12, 40), (18, 4), (18, 24), (19, 12)])
 def test_random_rotations(suite, tmp_path, n, count, dtype, tol):
-    status, worst, parts = _run(suite, tmp_path, n, _random(n, count, np.random.default_rng(n + count)), dtype)
+    status, worst, parts, inner = _run(suite, tmp_path, n, _random(n, count, np.random.default_rng(n + count)), dtype)
     assert status == 0 and worst < tol
     assert (parts > 0) == (n >= 18)
 
@@ -70,9 +70,9 @@ def test_molecular_strings(suite, tmp_path, orbitals, masks, dtype, tol):
     terms = prep.molecular_hamiltonian(h + h.T, g)
     terms = terms[np.isin(terms["x"], np.unique(terms["x"])[:masks])]
     rots = [(int(t["x"]), int(t["z"]), float(0.1 * t["coeff"])) for t in terms]
-    status, worst, parts = _run(suite, tmp_path, 2 * orbitals, rots, dtype)
+    status, worst, parts, inner = _run(suite, tmp_path, 2 * orbitals, rots, dtype)
     assert status == 0 and worst < tol
-    assert (parts > 0) == (orbitals == 9)
+    assert (parts > 0) == (inner > 0) == (orbitals == 9)
 
 
 @pytest.mark.parametrize("n", [12, 18])
@@ -86,11 +86,11 @@ def test_runs_of_one_mask(suite, tmp_path, n, parity):
             if x == 0 or bin(x & z).count("1") % 2 == parity:
                 rots.append((x, z, float(rng.uniform(-3.1, 3.1))))
                 count -= 1
-    status, worst, _ = _run(suite, tmp_path, n, rots, "c128")
+    status, worst, *_ = _run(suite, tmp_path, n, rots, "c128")
     assert status == 0 and worst < 1e-12
 
 
 def test_written_by_its_owner(suite, tmp_path):
     n = 18
-    status, worst, parts = _run(suite, tmp_path, n, _random(n, 10, np.random.default_rng(3)), "c128", ((1 << n) - 7,))
+    status, worst, parts, inner = _run(suite, tmp_path, n, _random(n, 10, np.random.default_rng(3)), "c128", ((1 << n) - 7,))
     assert status == 0 and worst < 1e-12
