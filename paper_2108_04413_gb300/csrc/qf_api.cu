@@ -2333,8 +2333,9 @@ qf_status apply_rotations(qf_state* st, const RotIn* list, size_t nrot) {
     }
     qf_status bf = flush_blocks();
     if (bf != QF_OK) return bf;
-    // A long run of one X mask; below kPhaseMin strings a sine and cosine a pair cost more
-    // FP64 operations (about 60 and one a string) than the rotations (four a string).
+    // A long run of one X mask; below kPhaseMin strings a sine and cosine a pair (about 60
+    // FP64 operations, and ten integer ones a string) cost more than the rotations (four FP64
+    // operations a string).
     // complex64 stays on the tiles: its rotations run at the FP32 rate.
     int len = run;
     if (r[i].x == 0)
@@ -2347,8 +2348,10 @@ qf_status apply_rotations(qf_state* st, const RotIn* list, size_t nrot) {
       pa.h = hibit(pa.x);
       pa.y = popc(pa.x & r[i].z) & 3;
       for (int k = 0; k < len; ++k) {
+        double th = r[i + k].th;
+        if (std::fabs(th) > qf::kPhaseMaxAngle) th = std::atan2(std::sin(th), std::cos(th));
         pa.z[k] = r[i + k].z;
-        pa.th[k] = ((popc(pa.x & r[i + k].z) - pa.y) & 2) ? -r[i + k].th : r[i + k].th;
+        pa.th[k] = ((popc(pa.x & r[i + k].z) - pa.y) & 2) ? -th : th;
       }
       // b: the reached indices with bit h cleared by x
       qf::Support span = sup;

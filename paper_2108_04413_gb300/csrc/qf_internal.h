@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include <string>
@@ -117,8 +118,23 @@ struct BlockPass {
   BlockRec b[kPassBlocks];
 };
 // A run of commuting rotations with one X mask: the rotation of a pair (b, b ^ x) by the
-// signed sum of their angles (see k_phase_run).
+// signed sum of their angles (see k_phase_run).  FP64 sums would lose digits as the angles
+// grow (256 angles within pi: 1.3e-13, within 1e6: 2.7e-8; a sine and cosine of each
+// rotation: 4e-15), so an angle is added as a whole number of 2^-62 turns, modulo 2^64:
+// exact sums of angles rounded to 7e-19.
 constexpr int kPhaseMax = 256, kPhaseMin = 24;
+constexpr double kPhaseMaxAngle = 1099511627776.0;  // 2^40: past it phase_turns runs out of digits
+inline __host__ __device__ uint64_t phase_turns(double th) {
+  constexpr double hi = 0x1.45f306dc9c883p-3, lo = -0x1.6b01ec5417056p-57;  // 1 / (2 pi) = hi + lo
+  const double p = th * hi;
+  const double e = fma(th, hi, -p) + th * lo;  // th / (2 pi) = p + e
+  const double unit = 4611686018427387904.0;
+  return (uint64_t)llrint((p - rint(p)) * unit) + (uint64_t)llrint(e * unit);
+}
+// The same angle in half turns, within +-1 (for sincospi).
+inline __host__ __device__ double phase_halves(uint64_t turns) {
+  return (double)(int64_t)(turns << 2) * (1.0 / 9223372036854775808.0);
+}
 struct PhaseArgs {
   int m;
   int h;       // highest set bit of x, -1 when x == 0
@@ -127,7 +143,7 @@ struct PhaseArgs {
   uint64_t x;
   Reached on;  // values of b, the pair's index with bit h clear
   uint64_t z[kPhaseMax];
-  double th[kPhaseMax];
+  double th[kPhaseMax];  // within kPhaseMaxAngle
 };
 // The tile of a block pass: a step costs a barrier more than it costs arithmetic, so the
 // large tile already from 2^5 tiles on.
