@@ -6,11 +6,28 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 
 #include "qf.h"
 
 namespace qf {
+
+// Raises Kernel's limit of dynamic shared memory on the current device, once on each: the
+// attribute belongs to the device, and a process may hold handles on several.
+template <auto Kernel>
+inline cudaError_t smem_limit(size_t bytes) {
+  static std::atomic<uint64_t> done{0};  // one bit a device; past 64, set on every call
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = dev < 64 ? 1ull << dev : 0ull;
+  if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(reinterpret_cast<const void*>(Kernel), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)bytes);
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+  return e;
+}
 
 // Largest tile / block shapes handled by the fused kernels.
 constexpr int kTileMaxRot = 32;   // rotations fused into one shared-memory tile pass

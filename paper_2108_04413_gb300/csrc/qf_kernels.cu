@@ -2046,11 +2046,6 @@ template <typename T>
 static cudaError_t tile_impl(void* psi, int n, const TileArgs& a, cudaStream_t s) {
   using V = typename Cx<T>::V;
   const size_t smem = (sizeof(V) << a.s) + (sizeof(uint64_t) << a.nhi);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(k_tile<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    attr_set = true;
-  }
   const uint64_t ntiles = 1ull << (n - a.s);
   int per_sm = 4;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tile<T>, 256, smem);
@@ -2065,9 +2060,8 @@ static cudaError_t tile_pass_t(void* psi, int n, const TileArgs& a, cudaStream_t
   using V = typename Cx<T>::V;
   constexpr int tiles_held = ADJ ? 2 : 1;
   const size_t smem = (sizeof(V) << S) * tiles_held + (ADJ ? a.m * 256 * sizeof(double) : 0);
-  constexpr int most = (int)((sizeof(V) << S) * tiles_held + (ADJ ? kTileAdjRot * 256 * sizeof(double) : 0));
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(k_tile_pass<T, S, ADJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  constexpr size_t most = (sizeof(V) << S) * tiles_held + (ADJ ? kTileAdjRot * 256 * sizeof(double) : 0);
+  const cudaError_t attr = smem_limit<k_tile_pass<T, S, ADJ>>(most);
   if (attr != cudaSuccess) return attr;
   if (ADJ && (a.m < 1 || a.m > kTileAdjRot)) return cudaErrorInvalidValue;
   const uint64_t tiles = 1ull << (n - S);
@@ -2153,8 +2147,7 @@ template <typename T, int S>
 static cudaError_t block_pass_t(void* psi, int n, const BlockPass& a, cudaStream_t s) {
   using V = typename Cx<T>::V;
   constexpr size_t smem = sizeof(V) << S;
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(k_block_pass<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t attr = smem_limit<k_block_pass<T, S>>(smem);
   if (attr != cudaSuccess) return attr;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)std::min<uint64_t>(1ull << (n - S), (uint64_t)sm_count() * (smem > 32768 ? 3 : 4)));
@@ -2364,8 +2357,7 @@ static cudaError_t expect_passes_t(const void* psi, int n, const ExpPass* passes
                                    unsigned* counter, double* out, cudaStream_t s) {
   using V = typename Cx<T>::V;
   constexpr size_t smem = sizeof(V) << PassTile<T>::S;
-  static const cudaError_t attr =  // thread-safe one-time initialisation
-      cudaFuncSetAttribute(k_expect_pass<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t attr = smem_limit<k_expect_pass<T>>(smem);
   if (attr != cudaSuccess) return attr;
   const uint64_t items = (uint64_t)npass << (n - PassTile<T>::S);
   const uint64_t grid = std::min<uint64_t>({items, (uint64_t)sm_count() * 3, (uint64_t)max_blocks});
@@ -2414,7 +2406,9 @@ static cudaError_t hpsi_tiled_e(const void* psi, void* lam, int n, bool realst, 
   // persistent grid: exactly the blocks that are resident at once (a partial
   // second wave would leave most SMs idle at the end)
   const auto k = realst ? k_hpsi_tiled<T, E, true> : k_hpsi_tiled<T, E, false>;
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t attr =
+      realst ? smem_limit<k_hpsi_tiled<T, E, true>>(smem) : smem_limit<k_hpsi_tiled<T, E, false>>(smem);
+  if (attr != cudaSuccess) return attr;
   int per_sm = 1;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem);
   if (per_sm < 1) per_sm = 1;

@@ -28,7 +28,6 @@
 #include <stdint.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "qf_internal.h"
 
@@ -2043,16 +2042,11 @@ static cudaError_t runs_t(void* psi, void* lam, const RunInfo* runs, int nruns, 
   // registers four of its wide CTAs would not fit an SM)
   constexpr bool kWide = MODE == 0 || (MODE == 3 && (DSW || sizeof(T) == 4));
   const bool wide = kWide && map != nullptr;
-  static std::once_flag once;  // allow the opt-in shared memory size, once per process
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    const int bytes = (int)run_smem_max<MODE, T>();
-    if (!DSW) attr = cudaFuncSetAttribute(k_sector_run<MODE, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if constexpr (kWide)
-      if (attr == cudaSuccess)
-        attr = cudaFuncSetAttribute(k_sector_run_wide<MODE, T, DSW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    bytes);
-  });
+  cudaError_t attr = cudaSuccess;  // allow the opt-in shared memory size
+  if constexpr (kWide)
+    if (wide) attr = smem_limit<k_sector_run_wide<MODE, T, DSW>>(run_smem_max<MODE, T>());
+  if constexpr (!DSW)
+    if (!wide) attr = smem_limit<k_sector_run<MODE, T>>(run_smem_max<MODE, T>());
   if (attr != cudaSuccess) return attr;
   for (int r = 0; r < nruns; ++r) {
     const RunInfo& R = runs[MODE != 0 ? nruns - 1 - r : r];
@@ -2141,8 +2135,7 @@ static cudaError_t overlaps_t(const void* psi, const RunInfo* runs, int nruns, c
                               double* partial, int pmax, double* out, const SecCompact& cm, cudaStream_t s) {
   using V = typename SCx<T>::V;
   constexpr int kMaxLists = 200 * 1024;  // the largest sector's strings: 2 x C(17, 8) words = 194480 bytes
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(k_pool_overlaps<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxLists);
+  const cudaError_t attr = smem_limit<k_pool_overlaps<T>>(kMaxLists);
   if (attr != cudaSuccess) return attr;
   PoolRuns pr;
   pr.slices = std::max(1, std::min(pmax, 8 * sm_count_s() / std::max(1, nblk)));
@@ -2246,13 +2239,14 @@ cudaError_t launch_sector_hpsi_direct(void* cpsi, qf_dtype dt, const SecSpace& s
   // partner ranks must fit 14 bits
   if (sp.cnt_o > (1u << 14)) return cudaErrorInvalidValue;
   const size_t smem = (size_t)std::max(1, sp.ko * (sp.no - sp.ko)) * 256 * sizeof(uint32_t);
+  constexpr size_t most = 64 * 256 * sizeof(uint32_t);
+  const cudaError_t attr = dt != QF_C128 ? smem_limit<k_sector_hpsi_direct<float, false>>(most)
+                           : split       ? smem_limit<k_sector_hpsi_direct<double, true>>(most)
+                                         : smem_limit<k_sector_hpsi_direct<double, false>>(most);
+  if (attr != cudaSuccess) return attr;
   const int prof_slot_ = prof_pre(QF_K_HPSI, s);
   const uint64_t items = (uint64_t)sp.cnt_e * sp.cnt_o;
   auto grid = [&](auto kernel) {  // every CTA the SMs hold at this shared-memory size
-    static std::once_flag once;
-    std::call_once(once, [&] {
-      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 256 * (int)sizeof(uint32_t));
-    });
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -2310,8 +2304,7 @@ size_t small_eval_smem(qf_dtype dt, uint32_t members, int ko, int no) {
 
 template <typename T, int NT>
 static cudaError_t small_eval_t(const SmallEval& a, int n_req, size_t smem, cudaStream_t s) {
-  static const cudaError_t attr =  // allow the opt-in shared memory size, once per process
-      cudaFuncSetAttribute(k_small_eval<T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmemCap);
+  const cudaError_t attr = smem_limit<k_small_eval<T, NT>>(kSmallSmemCap);  // the opt-in size
   if (attr != cudaSuccess) return attr;
   k_small_eval<T, NT><<<n_req, NT, smem, s>>>(a);
   return cudaGetLastError();
