@@ -11,6 +11,14 @@
 
 #include "qf.h"
 
+// Launchers that the planner does without where a host build of it (a test double of the
+// kernels) has none.  In the library they are ordinary symbols: it does not load without them.
+#ifdef __CUDACC__
+#define QF_OPTIONAL
+#else
+#define QF_OPTIONAL __attribute__((weak))
+#endif
+
 namespace qf {
 
 // Raises Kernel's limit of dynamic shared memory on the current device, once on each: the
@@ -450,28 +458,26 @@ cudaError_t launch_tile(void* psi, int n, qf_dtype dt, const TileArgs& a, cudaSt
 cudaError_t launch_sparse(void* psi, int n, qf_dtype dt, const SparseArgs& a, bool realst, cudaStream_t s);
 bool sparse_m_real(const SparseArgs& a);
 bool sparse_q_imag(const SparseArgs& a);
-// launch_sparse on the outside patterns of `on` (weak: see launch_check_support).
-__attribute__((weak)) cudaError_t launch_sparse_on(void* psi, int n, qf_dtype dt, const SparseArgs& a,
-                                                   const Reached& on, bool realst, cudaStream_t s);
-// Weak: see launch_check_support.
-__attribute__((weak)) cudaError_t launch_block_pass(void* psi, int n, qf_dtype dt, const BlockPass& a,
-                                                    cudaStream_t s);
-// complex128 only.  Weak: see launch_check_support.
-__attribute__((weak)) cudaError_t launch_phase_run(void* psi, int n, const PhaseArgs& a, cudaStream_t s);
+// launch_sparse on the outside patterns of `on`.
+QF_OPTIONAL cudaError_t launch_sparse_on(void* psi, int n, qf_dtype dt, const SparseArgs& a,
+                                         const Reached& on, bool realst, cudaStream_t s);
+QF_OPTIONAL cudaError_t launch_block_pass(void* psi, int n, qf_dtype dt, const BlockPass& a,
+                                          cudaStream_t s);
+// complex128 only.
+QF_OPTIONAL cudaError_t launch_phase_run(void* psi, int n, const PhaseArgs& a, cudaStream_t s);
 // *dense = 1 when an amplitude outside s is nonzero (dense zeroed on the stream before).
-// Weak: a build of the planner without the kernels visits every tile.
-__attribute__((weak)) cudaError_t launch_check_support(const void* psi, int n, qf_dtype dt, const Support& s,
-                                                       unsigned* dense, cudaStream_t stream);
+QF_OPTIONAL cudaError_t launch_check_support(const void* psi, int n, qf_dtype dt, const Support& s,
+                                             unsigned* dense, cudaStream_t stream);
 // <psi|H|psi> for the grouped plan; writes the sum into out[0] (device).
 cudaError_t launch_expect(const void* psi, int n, qf_dtype dt, const ExpGroup* groups, int ngroups,
                           const ExpChunk* chunks, double* partials, unsigned* counter, double* out,
                           int nblocks, cudaStream_t s);
 // The same for groups gathered into passes (n >= PassTile::S): tabs are the plan's
-// ExpChunks.  Weak: a build of the planner without the kernels takes launch_expect.
-__attribute__((weak)) cudaError_t launch_expect_passes(const void* psi, int n, qf_dtype dt, const ExpPass* passes,
-                                                       int npass, const PassGroup* groups, const PassChunk* chunks,
-                                                       const ExpChunk* tabs, double* partials, int max_blocks,
-                                                       unsigned* counter, double* out, cudaStream_t s);
+// ExpChunks.
+QF_OPTIONAL cudaError_t launch_expect_passes(const void* psi, int n, qf_dtype dt, const ExpPass* passes,
+                                             int npass, const PassGroup* groups, const PassChunk* chunks,
+                                             const ExpChunk* tabs, double* partials, int max_blocks,
+                                             unsigned* counter, double* out, cudaStream_t s);
 // lam = H psi, out[0] = Re <psi|lam>, out[1] = <psi|psi>; partials holds 2 * nblocks doubles.
 cudaError_t launch_hpsi(const void* psi, void* lam, int n, qf_dtype dt, const ExpGroup* groups, int ngroups,
                         const ExpChunk* chunks, double* partials, unsigned* counter, double* out, int nblocks,
