@@ -1763,6 +1763,7 @@ __global__ void __launch_bounds__(256, 4) k_sector_hpsi_direct(T* st, SecDirect 
 constexpr int kSmallStepMax = 512;       // threads of the block steps, at most
 constexpr int kSmallRing = 8;            // steps whose map words and coefficients sit in shared memory
 constexpr int kSmallBatch = 8;           // steps whose overlaps are summed together
+constexpr size_t kSmallStepBytes = kSmallRing * 2 * sizeof(uint32_t) + kSmallBatch * 2 * 8;  // per step thread
 constexpr size_t kSmallSmemMax = 200u * 1024u;  // psi, lambda and the beta-single lists of 256 threads
 constexpr size_t kSmallSmemCap = 224u * 1024u;  // with all else (static shared memory: under 3 KB of 227)
 
@@ -1809,7 +1810,8 @@ __device__ __forceinline__ void step_barrier(int n) { asm volatile("bar.sync 1, 
 // step thread), the overlaps of kSmallBatch steps (each step thread's), then the H psi
 // step's beta-single lists, which share the room of the two before (the sweeps come
 // before and after it).
-template <typename T, int NT>
+// LISTED: the steps' item counts sit in shared memory (2 bytes a block).
+template <typename T, int NT, bool LISTED>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_small_eval(SmallEval a) {
   const int ST = a.step_threads, NW = ST / 32;  // threads and warps of the block steps
   extern __shared__ __align__(16) unsigned char dsm[];
@@ -1821,14 +1823,16 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small_eval(SmallEval a) {
   T* ps = reinterpret_cast<T*>(dsm);
   T* lm = ps + M;
   uint16_t* sn = reinterpret_cast<uint16_t*>(dsm + align16(2 * (size_t)M * sizeof(T)));  // every block's items
-  unsigned char* room = reinterpret_cast<unsigned char*>(sn) + align16(nb * sizeof(uint16_t));
+  unsigned char* room = reinterpret_cast<unsigned char*>(sn) + (LISTED ? align16(nb * sizeof(uint16_t)) : 0);
   uint32_t* mw = reinterpret_cast<uint32_t*>(room);
   StepSum<T>* red = reinterpret_cast<StepSum<T>*>(mw + kSmallRing * 2 * ST);
   uint32_t* bsl = reinterpret_cast<uint32_t*>(room);
   const T* cf = static_cast<const T*>(a.coef) + (size_t)blockIdx.x * a.nblk * kSmallCoef;
   double* out = a.out + (size_t)blockIdx.x * (a.nblk + 2);
   fill_binom(C);
-  for (int b = tid; b < nb; b += NT) sn[b] = (uint16_t)__ldg(&a.steps[b].y);
+  if (LISTED)
+    for (int b = tid; b < nb; b += NT) sn[b] = (uint16_t)__ldg(&a.steps[b].y);
+  auto items = [&](int b) -> uint32_t { return LISTED ? sn[b] : __ldg(&a.steps[b].y); };
   for (uint32_t m = tid; m < M; m += NT) ps[m] = (m == a.c0) ? T(1) : T(0);
   // the block steps in order (REV: from the last block, with the inverse's
   // coefficients and the overlaps); item(i0, i1, m, class, sum) handles one item
@@ -1839,11 +1843,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small_eval(SmallEval a) {
     auto blk = [&](int s) { return REV ? nb - 1 - s : s; };
     // map offsets of the step to load and of the current step
     uint32_t lo = 0, so = 0;
-    if (REV && nb > 0) lo = so = __ldg(&a.steps[nb - 1].x) + sn[nb - 1];
+    if (REV && nb > 0) lo = so = __ldg(&a.steps[nb - 1].x) + items(nb - 1);
     auto load = [&](int s) {  // one step's loads are one copy group
       if (s < nb) {
         const int slot = s & (kSmallRing - 1);
-        const uint32_t n = sn[blk(s)];
+        const uint32_t n = items(blk(s));
         if (REV) lo -= n;
         uint32_t* w = mw + slot * 2 * ST + tid;
         if ((uint32_t)tid < n) cp_async_small(w, a.map + lo + tid);
@@ -1861,7 +1865,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small_eval(SmallEval a) {
       for (int r = warp; r < cnt; r += NW) {
         const int q = s - cnt + r;
         const StepSum<T>* row = red + (q & (2 * kSmallBatch - 1)) * ST;
-        const uint32_t n = sn[blk(q)];
+        const uint32_t n = items(blk(q));
         StepSum<T> v;
         for (uint32_t j = lane; j < (uint32_t)ST && (j & ~31u) < n; j += 32) v.add(row[j]);
         int e;
@@ -1873,7 +1877,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small_eval(SmallEval a) {
     for (int s = 0; s < nb; ++s) {
       const int slot = s & (kSmallRing - 1);
       load(s + D);  // into the slot of step s - 1
-      const uint32_t n = sn[blk(s)];
+      const uint32_t n = items(blk(s));
       if (REV) so -= n;
       const T* c = cw[slot];
       StepSum<T> acc;
@@ -2302,11 +2306,11 @@ size_t small_eval_smem(qf_dtype dt, uint32_t members, int ko, int no) {
   return members < kSmallMaxMembers && b <= kSmallSmemMax ? b : 0;
 }
 
-template <typename T, int NT>
+template <typename T, int NT, bool LISTED>
 static cudaError_t small_eval_t(const SmallEval& a, int n_req, size_t smem, cudaStream_t s) {
-  const cudaError_t attr = smem_limit<k_small_eval<T, NT>>(kSmallSmemCap);  // the opt-in size
+  const cudaError_t attr = smem_limit<k_small_eval<T, NT, LISTED>>(kSmallSmemCap);  // the opt-in size
   if (attr != cudaSuccess) return attr;
-  k_small_eval<T, NT><<<n_req, NT, smem, s>>>(a);
+  k_small_eval<T, NT, LISTED><<<n_req, NT, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -2320,28 +2324,34 @@ cudaError_t launch_small_eval(const SmallEval& req, qf_dtype dt, int n_req, cuda
   // two requests share one; 256 where the lists need the room.  The steps by as many
   // as a typical block has items (a step's fixed work grows with its warps).
   const size_t real = dt == QF_C128 ? sizeof(double) : sizeof(float);
-  const size_t fixed = align16(2 * (size_t)members * real) + align16(a.nblk * sizeof(uint16_t));
-  int nt = n_req <= sm_count_s() ? 1024 : 512;
+  const size_t state = align16(2 * (size_t)members * real);
+  const size_t list = (size_t)std::max(1, a.ko * (a.d.no - a.ko)) * sizeof(uint32_t);  // a thread's
   size_t smem = 0;
-  for (;; nt /= 2) {
-    const size_t lists = (size_t)std::max(1, a.ko * (a.d.no - a.ko)) * nt * sizeof(uint32_t);
+  auto fits = [&](int nt, size_t counts) {
     for (a.step_threads = std::min({nt, kSmallStepMax, std::max(128, (req.step_threads + 127) / 128 * 128)});;
          a.step_threads -= 32) {
-      const size_t steps = (size_t)a.step_threads * (kSmallRing * 2 * sizeof(uint32_t) + kSmallBatch * 2 * 8);
-      smem = fixed + std::max(lists, steps);
+      smem = state + counts + std::max(list * nt, a.step_threads * kSmallStepBytes);
       if (smem <= kSmallSmemCap || a.step_threads == 96) break;
     }
-    if (smem <= kSmallSmemCap || nt == 256) break;
-  }
-  if (smem > kSmallSmemCap) return cudaErrorInvalidValue;
+    return smem <= kSmallSmemCap;
+  };
+  const size_t counts = align16(a.nblk * sizeof(uint16_t));
+  int nt = n_req <= sm_count_s() ? 1024 : 512;
+  while (nt >= 256 && !fits(nt, counts)) nt /= 2;
+  // thousands of blocks beside a sector that nearly fills the CTA: their item counts are
+  // read from global memory (always reading them there: 14 qubits, 32 requests 426 -> 439 us)
+  static_assert(kSmallSmemMax + 96 * kSmallStepBytes <= kSmallSmemCap, "what small_eval_smem admits fits");
+  if (nt < 256 && !fits(256, 0)) return cudaErrorInvalidValue;
   const int prof_slot_ = prof_pre(QF_K_SPARSE, s);
   const cudaError_t e =
-      dt == QF_C128 ? (nt == 1024  ? small_eval_t<double, 1024>(a, n_req, smem, s)
-                       : nt == 512 ? small_eval_t<double, 512>(a, n_req, smem, s)
-                                   : small_eval_t<double, 256>(a, n_req, smem, s))
-                    : (nt == 1024  ? small_eval_t<float, 1024>(a, n_req, smem, s)
-                       : nt == 512 ? small_eval_t<float, 512>(a, n_req, smem, s)
-                                   : small_eval_t<float, 256>(a, n_req, smem, s));
+      dt == QF_C128 ? (nt == 1024  ? small_eval_t<double, 1024, true>(a, n_req, smem, s)
+                       : nt == 512 ? small_eval_t<double, 512, true>(a, n_req, smem, s)
+                       : nt == 256 ? small_eval_t<double, 256, true>(a, n_req, smem, s)
+                                   : small_eval_t<double, 256, false>(a, n_req, smem, s))
+                    : (nt == 1024  ? small_eval_t<float, 1024, true>(a, n_req, smem, s)
+                       : nt == 512 ? small_eval_t<float, 512, true>(a, n_req, smem, s)
+                       : nt == 256 ? small_eval_t<float, 256, true>(a, n_req, smem, s)
+                                   : small_eval_t<float, 256, false>(a, n_req, smem, s));
   count_launch();
   prof_post(prof_slot_, s);
   return e;
