@@ -245,6 +245,7 @@ struct qf_state {
   void* d_small = nullptr;
   size_t small_cap = 0;
   uint64_t small_key = 0;
+  uint64_t small_none = 0;  // a plan and sector whose item map did not fit
   int small_items = 0;      // items of an average block
   // Per block of that plan: its composite at parameter t is cos(kap t) on the diagonal
   // and s01 / s10 sin(kap t) off it, per sign class, and the generator's entry q01
@@ -335,6 +336,7 @@ void trim_plans(qf_state* st) {
     st->parts_key = 0;  // descriptors on the device are re-uploaded by their next user
     st->map_key = 0;
     st->pool_key = 0;
+    st->small_key = st->small_none = 0;
   }
 }
 
@@ -2710,7 +2712,7 @@ static qf_status energy_grad_impl(qf_state* st, uint64_t det, const qf_arot* ans
       ait = st->ansatz_plans.end();
       st->parts_key = 0;
       st->map_key = 0;
-      st->small_key = 0;
+      st->small_key = st->small_none = 0;
     }
   }
   // a cached plan's rotations had their masks checked when it was built
@@ -3198,17 +3200,22 @@ qf_status ensure_host(void** p, size_t* cap, size_t bytes, const char* what) {
 }
 
 // The item map of a small sector's forward blocks (qf::SmallEval): every block's items
-// in the sweeps' order (alpha outside strings, then beta ones, both colex).
-void small_itemmap(const std::vector<qf::SecBlk>& g, const qf::SecSpace& sp, std::vector<uint2>* steps,
+// in the sweeps' order (alpha outside strings, then beta ones, both colex).  False, and
+// nothing made, when it would take more than kSmallMapWords.
+constexpr uint64_t kSmallMapWords = 1ull << 28;  // 1 GB, as the part-local sweeps' maps
+bool small_itemmap(const std::vector<qf::SecBlk>& g, const qf::SecSpace& sp, std::vector<uint2>* steps,
                    std::vector<uint32_t>* map) {
+  uint64_t off = 0;
+  for (const qf::SecBlk& b : g) off += (uint64_t)b.cnt_e * b.cnt_o;
+  if (off > kSmallMapWords) return false;
+  map->resize(std::max<uint64_t>(1, off));
   steps->resize(g.size());
-  uint32_t off = 0;
+  off = 0;
   for (size_t b = 0; b < g.size(); ++b) {
-    (*steps)[b].x = off;
+    (*steps)[b].x = (uint32_t)off;
     (*steps)[b].y = g[b].cnt_e * g[b].cnt_o;
     off += (*steps)[b].y;
   }
-  map->resize(std::max<uint32_t>(1, off));
   qf::HostPool::get().parallel_for(g.size(), 8, [&](size_t b) {
     const qf::SecBlk& B = g[b];
     // one spin's outside strings: the ranks with either pattern, and the class bits
@@ -3239,6 +3246,7 @@ void small_itemmap(const std::vector<qf::SecBlk>& g, const qf::SecSpace& sp, std
       for (const Side& o : side[1])
         *w++ = (e.r0 * sp.cnt_o + o.r0) | ((e.r1 * sp.cnt_o + o.r1) << 15) | ((e.cls ^ o.cls) << 30);
   });
+  return true;
 }
 
 // A block's closed form (see compose_sparse): kap, the signed sum of its rotations'
@@ -3330,6 +3338,7 @@ qf_status multi_small(qf_state* st, uint64_t det, const qf_arot* ansatz, size_t 
   if (!finite.load()) return fail(QF_EINVAL, "theta is not finite");
   // the forward blocks' geometry for this sector, on the device once
   const uint64_t skey = content_key(nullptr, 0, ait->first ^ ((uint64_t)na << 40) ^ ((uint64_t)nbeta << 48)) | 1ull;
+  if (st->small_none == skey) return QF_OK;  // its map did not fit before: row by row
   if (st->small_key != skey) {
     for (const auto& b : blocks) {  // the reverse reads the forward geometry with the inverse's coefficients
       if (!b.sparse || b.fwd.nr != 2 || b.inv.nr != 2 || b.fwd.nzc != b.inv.nzc) return QF_OK;
@@ -3346,12 +3355,14 @@ qf_status multi_small(qf_state* st, uint64_t det, const qf_arot* ansatz, size_t 
     }
     std::vector<uint2> steps;
     std::vector<uint32_t> map;
-    small_itemmap(g, sp, &steps, &map);
     st->small_key = 0;
-    qf_status bs = ensure_buf(&st->d_small, &st->small_cap,
-                              nblk * (sizeof(qf::SecBlk) + sizeof(uint2)) + map.size() * sizeof(uint32_t),
-                              "small-request blocks");
-    if (bs != QF_OK) return bs;
+    if (!small_itemmap(g, sp, &steps, &map) ||
+        ensure_buf(&st->d_small, &st->small_cap,
+                   nblk * (sizeof(qf::SecBlk) + sizeof(uint2)) + map.size() * sizeof(uint32_t),
+                   "small-request blocks") != QF_OK) {
+      st->small_none = skey;
+      return QF_OK;
+    }
     char* d = static_cast<char*>(st->d_small);
     QF_CUDA(h2d(d, g.data(), nblk * sizeof(qf::SecBlk), st->stream));
     d += nblk * sizeof(qf::SecBlk);
@@ -3574,6 +3585,7 @@ qf_status qf_state_clear_plans(qf_state* st) {
   st->plans.clear();
   st->ansatz_plans.clear();
   st->parts_key = st->pool_key = st->map_key = 0;  // descriptors on the device belong to no plan now
+  st->small_key = st->small_none = 0;
   return QF_OK;
 }
 
