@@ -65,10 +65,15 @@ TABLE_BYTES_PER_TERM = 512
 RUN_BYTES_PER_EXCITATION = 1536
 LOG_MAX_BYTES = 16 << 30
 MAP_MAX_BYTES = 1 << 30
+# Grouped requests (qf_energy_grad_multi): sectors of which psi and lambda fit a CTA,
+# the block geometries, and each row's composites (36 reals) and overlap per excitation.
+GROUPED_SECTOR_BYTES = 200 << 10
+GROUPED_BYTES_PER_EXCITATION = 512
+GROUPED_REALS_PER_ROW = 36
 
 
 def footprint_bytes(n: int, dtype: str, det: Optional[int] = None, ansatz: Optional[np.ndarray] = None,
-                    n_terms: int = 0) -> int:
+                    n_terms: int = 0, rows: int = 1) -> int:
     """Device bytes a resident system holds, an upper bound: psi and lambda
     (2 * 2^n amplitudes), the handle's work buffers and its Pauli-sum plan tables
     (n_terms terms).  Given the determinant and the ansatz, also the sector
@@ -76,7 +81,9 @@ def footprint_bytes(n: int, dtype: str, det: Optional[int] = None, ansatz: Optio
     pair per (member pair, excitation) item, at most 16 GB), its item maps (at
     most one 4-byte word per item, at most 1 GB) and its run descriptors: an
     excitation whose flips cover sa alpha and sb beta spin orbitals, half of each
-    occupied, moves C(ne - sa, na - sa/2) * C(no - sb, nb - sb/2) items."""
+    occupied, moves C(ne - sa, na - sa/2) * C(no - sb, nb - sb/2) items.  rows: the
+    most requests one grouped call takes; from two on, also that call's item map and
+    records (for sectors small enough to be grouped)."""
     from math import comb
 
     size = 16 if dtype == "c128" else 8
@@ -96,6 +103,9 @@ def footprint_bytes(n: int, dtype: str, det: Optional[int] = None, ansatz: Optio
         ka, kb = na - sa // 2, nb - sb // 2
         if 0 <= ka <= ne - sa and 0 <= kb <= no - sb:
             items += comb(ne - sa, ka) * comb(no - sb, kb)
+    if rows > 1 and members * size <= GROUPED_SECTOR_BYTES:
+        per_row = len(flips) * (GROUPED_REALS_PER_ROW * size // 2 + 8) + 16
+        total += min(items * 4, MAP_MAX_BYTES) + GROUPED_BYTES_PER_EXCITATION * len(flips) + rows * per_row
     return (total + 2 * members * size + min(items * size, LOG_MAX_BYTES) + min(items * 4, MAP_MAX_BYTES) +
             RUN_BYTES_PER_EXCITATION * len(flips))
 
@@ -175,7 +185,8 @@ class Server:
         fp = self._fp.get(key)
         if fp is None:
             sysm = self.systems[key]
-            fp = self._fp[key] = footprint_bytes(sysm.n, self.dtype, sysm.det, sysm.ansatz, len(sysm.terms))
+            rows = self.batch if sysm.n <= self.batch_qubits else 1
+            fp = self._fp[key] = footprint_bytes(sysm.n, self.dtype, sysm.det, sysm.ansatz, len(sysm.terms), rows)
         return fp
 
     # -- submission
