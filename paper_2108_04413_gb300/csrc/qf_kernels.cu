@@ -1159,7 +1159,7 @@ template <> struct PassAcc<float> {
     h = t;
   }
   __device__ __forceinline__ double take() {
-    const double v = (double)h + (double)l;
+    const double v = (double)h + (double)(isfinite(h) ? l : 0.f);  // TwoSum's error of an infinity is a NaN
     h = l = 0.f;
     return v;
   }
