@@ -1784,6 +1784,8 @@ template <> struct StepSum<double> {
   __device__ __forceinline__ void add(double d) { v += d; }
   __device__ __forceinline__ void add(const StepSum& o) { v += o.v; }
   __device__ __forceinline__ long long warp(int* e) const { return warp_sum_fixed(v, e); }
+  __device__ __forceinline__ bool finite() const { return isfinite(v); }
+  __device__ __forceinline__ double value() const { return v; }
 };
 template <> struct StepSum<float> {
   float2 v = make_float2(0.f, 0.f);
@@ -1801,6 +1803,8 @@ template <> struct StepSum<float> {
     r.x = two_sum(v.x, v.y, &r.y);
     return warp_sum_fixed_ds(r, e);
   }
+  __device__ __forceinline__ bool finite() const { return isfinite(v.x); }
+  __device__ __forceinline__ double value() const { return (double)v.x + (double)(finite() ? v.y : 0.f); }
 };
 
 // Barrier of the CTA's first n threads (whole warps).
@@ -1870,7 +1874,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_small_eval(SmallEval a) {
         for (uint32_t j = lane; j < (uint32_t)ST && (j & ~31u) < n; j += 32) v.add(row[j]);
         int e;
         const long long t = v.warp(&e);
-        const double d = warp_fixed_to_double(lane == 0 ? t : 0ll, lane == 0 ? e : 0);
+        double d = warp_fixed_to_double(lane == 0 ? t : 0ll, lane == 0 ? e : 0);
+        if (!__all_sync(0xffffffffu, v.finite())) {  // the integer scale has no infinity and no NaN
+          d = v.value();
+          for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
+        }
         if (lane == 0) out[blk(q)] = d;
       }
     };
