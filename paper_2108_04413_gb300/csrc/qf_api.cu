@@ -80,6 +80,7 @@ struct ExpPlan {
   std::vector<qf_term> terms;        // the plan's terms (compared on every cache hit; tiled tables)
   std::vector<qf::ExpGroup> groups;  // host copies for the expectation passes
   std::vector<uint64_t> chunk_z;     // kChunkTerms masks per expectation chunk
+  double weight = 0.0;   // sum of |coeff|
   bool has_odd = false;  // some term has an odd number of Y letters (imaginary phase)
   uint64_t last_use = 0; // the handle's call count at the plan's last use (least recently used goes first)
   // direct sector H|psi> tables (qf::SecDirect): 0 not tried yet, 1 built, -1 the
@@ -732,6 +733,7 @@ qf_status get_plan(qf_state* st, const qf_term* terms, size_t nt, const ExpPlan*
     QF_CUDA(cudaStreamSynchronize(st->stream));
   }
   p.terms.assign(terms, terms + nt);
+  for (const qf_term& t : p.terms) p.weight += std::fabs(t.coeff);
   p.chunk_z.reserve(ech.size() * qf::kChunkTerms);
   for (const qf::ExpChunk& c : ech) p.chunk_z.insert(p.chunk_z.end(), c.z, c.z + qf::kChunkTerms);
   p.groups = std::move(groups);
@@ -3104,6 +3106,11 @@ static qf_status energy_grad_impl(qf_state* st, uint64_t det, const qf_arot* ans
   // reverse sweep; psi and lam share one scale
   std::vector<double> s2(blocks.size());
   double sc = s_fwd;
+  // Reverse passes of complex64 take the overlaps' products in FP32 (DotAcc), which hold any
+  // conj(lambda) psi, at most weight / scale^2 with a scale of 2^-31 or more, only for a
+  // weight below 2^60 (and their rounding errors above 2^-60): past these, rotation by
+  // rotation with FP64 products.
+  const bool tiles_back = n >= qf::kTileSmall && (st->dt == QF_C128 || !p || (p->weight < 0x1p60 && p->weight > 0x1p-60));
   // psi and lambda = H psi are both real when psi is real and H has no odd-Y term
   bool both_real = st->real && (!p || !p->has_odd);
   for (size_t bi = blocks.size(); bi-- > 0;) {
@@ -3116,7 +3123,7 @@ static qf_status energy_grad_impl(qf_state* st, uint64_t det, const qf_arot* ans
       both_real = both_real && rm;
     } else {
       int most = 1;
-      while (n >= qf::kTileSmall && most < qf::kTileAdjRot && (size_t)most <= bi && !blocks[bi - most].sparse) ++most;
+      while (tiles_back && most < qf::kTileAdjRot && (size_t)most <= bi && !blocks[bi - most].sparse) ++most;
       uint64_t uni = 0;
       RotIn back[qf::kTileAdjRot];  // the inverse rotations, last block first
       for (int k = 0; k < most; ++k) {
