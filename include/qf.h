@@ -209,7 +209,7 @@ void qf_transfer_bytes(int reset, uint64_t* h2d_bytes, uint64_t* d2h_bytes);
 /* Kernel kinds for the timing calls below. */
 #define QF_K_SET 1u          /* basis preparation, scale folding */
 #define QF_K_ROT 2u          /* unfused rotation (one pair sweep) */
-#define QF_K_TILE 4u         /* fused rotations in shared-memory tiles */
+#define QF_K_TILE 4u         /* fused rotations (tiles, runs of one X mask) and the check of a state they may read in part */
 #define QF_K_SPARSE 8u       /* sparse composite block */
 #define QF_K_EXPECT 16u      /* grouped expectation value */
 #define QF_K_HPSI 32u        /* H|psi> with <psi|H|psi> and <psi|psi> */

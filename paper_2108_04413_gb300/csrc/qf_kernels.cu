@@ -2118,10 +2118,12 @@ cudaError_t launch_check_support(const void* psi, int n, qf_dtype dt, const Supp
   }
   const uint64_t N = 1ull << n;
   const unsigned g = grid_for(N, 8);
+  const int prof_slot_ = prof_pre(QF_K_TILE, stream);
   if (dt == QF_C128)
     k_check_support<<<g, 256, 0, stream>>>(static_cast<const double2*>(psi), N, a, dense);
   else
     k_check_support<<<g, 256, 0, stream>>>(static_cast<const float2*>(psi), N, a, dense);
+  prof_post(prof_slot_, stream);
   count_launch();
   return cudaGetLastError();
 }
