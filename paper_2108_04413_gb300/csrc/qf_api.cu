@@ -231,7 +231,7 @@ struct qf_state {
   size_t runblk_cap = 0;
   void* d_idx = nullptr;     // residual read-out indices
   size_t idx_cap = 0;
-  void* d_poolblk = nullptr; // operator-pool run descriptors (blocks, parts, strings)
+  void* d_poolblk = nullptr; // operator-pool block descriptors
   size_t poolblk_cap = 0;
   uint64_t pool_key = 0;     // the pool plan and sector whose descriptors sit in d_poolblk
   void* d_map = nullptr;     // item maps of the part-local sweeps (RunPart::mapbase)
@@ -2980,25 +2980,20 @@ static qf_status energy_grad_impl(qf_state* st, uint64_t det, const qf_arot* ans
     double* d_pool = st->d_out + nblk + 2 + 2 * n_dets;
     if (pp) {  // every pool operator's overlap with the final (psi, lambda): nothing rotated
       const SectorRuns& pr = pp->runs;
-      const size_t pblk = pr.blks.size() * sizeof(qf::RunBlk), ppart = pr.parts.size() * sizeof(qf::RunPart);
+      const size_t pblk = pr.blks.size() * sizeof(qf::RunBlk);
       const void* pbefore = st->d_poolblk;
-      bs = ensure_buf(&st->d_poolblk, &st->poolblk_cap, pblk + ppart + pr.strs.size() * sizeof(uint16_t),
-                      "pool run descriptors");
+      bs = ensure_buf(&st->d_poolblk, &st->poolblk_cap, pblk, "pool run descriptors");
       if (bs != QF_OK) return bs;
       const uint64_t key =
           content_key(nullptr, 0, pkey0 ^ ((uint64_t)na << 40) ^ ((uint64_t)nbeta << 48) ^ cap) | 1ull;
       if (st->pool_key != key || st->d_poolblk != pbefore) {  // zero angle: the descriptors never change
-        char* base = static_cast<char*>(st->d_poolblk);
-        QF_CUDA(h2d(base, pr.blks.data(), pblk, st->stream));
-        QF_CUDA(h2d(base + pblk, pr.parts.data(), ppart, st->stream));
-        if (!pr.strs.empty()) QF_CUDA(h2d(base + pblk + ppart, pr.strs.data(), pr.strs.size() * 2, st->stream));
+        QF_CUDA(h2d(st->d_poolblk, pr.blks.data(), pblk, st->stream));
         st->pool_key = key;
       }
-      const char* base = static_cast<const char*>(st->d_poolblk);
       QF_CUDA(qf::launch_sector_overlaps(
-          cpsi, st->dt, pr.runs.data(), (int)pr.runs.size(), reinterpret_cast<const qf::RunPart*>(base + pblk),
-          reinterpret_cast<const qf::RunBlk*>(base) + npool_blk, (int)npool_blk, st->d_sec_partial, pr.pmax, d_pool,
-          cm, pr.strs.empty() ? nullptr : reinterpret_cast<const uint16_t*>(base + pblk + ppart), st->stream));
+          cpsi, st->dt, pr.runs.data(), (int)pr.runs.size(), nullptr,
+          static_cast<const qf::RunBlk*>(st->d_poolblk) + npool_blk, (int)npool_blk, st->d_sec_partial, pr.pmax, d_pool,
+          cm, nullptr, st->stream));
     }
     if (need_reverse)
       QF_CUDA(qf::launch_sector_runs(cpsi, clam, st->dt, true, lreal, rs.runs.data(), nruns, d_parts, d_blks + nblk,

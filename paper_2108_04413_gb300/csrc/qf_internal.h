@@ -530,7 +530,8 @@ cudaError_t launch_sector_runs(void* psi, void* lam, qf_dtype dt, bool adj, bool
                                const uint32_t* map, bool ds, bool dss, cudaStream_t s);
 // Overlaps only: out[b] = Im <lam|Q_b|psi> of every block b on the same compact
 // state (psi real parts, lam real parts in psi's imaginary slots); nothing is
-// rotated.  Same descriptors as launch_sector_runs; partial holds nblk * pmax values.
+// rotated.  Runs and blocks as launch_sector_runs takes them; it reads no parts and no
+// strings (they may be NULL); partial holds nblk * pmax values.
 cudaError_t launch_sector_overlaps(void* psi, qf_dtype dt, const RunInfo* runs, int nruns, const RunPart* parts,
                                   const RunBlk* blks, int nblk, double* partial, int pmax, double* out,
                                   const SecCompact& cm, const uint16_t* strs, cudaStream_t s);

@@ -1452,7 +1452,8 @@ __global__ void __launch_bounds__(256, 2) k_hpsi_tiled(const typename Cx<T>::V* 
                                                     const typename WTab<T>::C* __restrict__ chunks,
                                                     double* partials, unsigned* counter, double* out) {
   using V = typename Cx<T>::V;
-  constexpr int TB = (E == 1) ? 8 : (E == 2) ? 9 : (E == 4) ? 10 : (E == 8) ? 11 : 12;
+  static_assert(E == 4 || E == 8, "tiles of 2^10 and 2^11 amplitudes");
+  constexpr int TB = E == 4 ? 10 : 11;
   constexpr int KB = TB - 8;  // bits of k
   constexpr unsigned E16 = 16 / sizeof(V);
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1529,9 +1530,9 @@ __global__ void __launch_bounds__(256, 2) k_hpsi_tiled(const typename Cx<T>::V* 
         // the first table initialises D (no add of zero), later tables add to it
         for (int c = 0; c < G.nchunk; ++c) {
           const typename WTab<T>::C* W = chunks + G.chunk0 + c;
-          unsigned ith = 0, col[KB > 0 ? KB : 1];
+          unsigned ith = 0, col[KB];
 #pragma unroll
-          for (int j = 0; j < (KB > 0 ? KB : 1); ++j) col[j] = 0;
+          for (int j = 0; j < KB; ++j) col[j] = 0;
 #pragma unroll
           for (int q = 0; q < kWideTerms; ++q) {
             const uint64_t z = W->z[q];
@@ -2397,40 +2398,40 @@ cudaError_t launch_hpsi(const void* psi, void* lam, int n, qf_dtype dt, const Ex
   return cudaGetLastError();
 }
 
-template <typename T, int E>
-static cudaError_t hpsi_tiled_e(const void* psi, void* lam, int n, bool realst, const HClass* classes, int nclasses,
+template <typename T, int E, bool REALST>
+static cudaError_t hpsi_tiled_e(const void* psi, void* lam, int n, const HClass* classes, int nclasses,
                                 const HGroup* groups, const void* chunks, double* partials, unsigned* counter,
                                 double* out, int nblocks, cudaStream_t s) {
   using V = typename Cx<T>::V;
   using C = typename WTab<T>::C;
   const size_t smem = sizeof(V) * 256 * E * kHpsiStages;
-  const uint64_t ntiles = 1ull << (n - (8 + (E == 1 ? 0 : E == 2 ? 1 : E == 4 ? 2 : E == 8 ? 3 : 4)));
+  const uint64_t ntiles = (1ull << n) / (256 * E);
+  const cudaError_t attr = smem_limit<k_hpsi_tiled<T, E, REALST>>(smem);
+  if (attr != cudaSuccess) return attr;
   // persistent grid: exactly the blocks that are resident at once (a partial
   // second wave would leave most SMs idle at the end)
-  const auto k = realst ? k_hpsi_tiled<T, E, true> : k_hpsi_tiled<T, E, false>;
-  const cudaError_t attr =
-      realst ? smem_limit<k_hpsi_tiled<T, E, true>>(smem) : smem_limit<k_hpsi_tiled<T, E, false>>(smem);
-  if (attr != cudaSuccess) return attr;
   int per_sm = 1;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hpsi_tiled<T, E, REALST>, 256, smem);
   if (per_sm < 1) per_sm = 1;
   uint64_t cap = (uint64_t)sm_count() * (uint64_t)per_sm;
   if (cap > (uint64_t)nblocks) cap = (uint64_t)nblocks;
   unsigned g = (unsigned)std::min<uint64_t>(ntiles, cap);
-  k<<<g, 256, smem, s>>>(static_cast<const V*>(psi), static_cast<V*>(lam), n, classes, nclasses, groups,
-                         static_cast<const C*>(chunks), partials, counter, out);
+  k_hpsi_tiled<T, E, REALST><<<g, 256, smem, s>>>(static_cast<const V*>(psi), static_cast<V*>(lam), n, classes,
+                                                  nclasses, groups, static_cast<const C*>(chunks), partials, counter,
+                                                  out);
   return cudaGetLastError();
 }
 
+// Tiles of 2^10 amplitudes, and of 2^11 for a real state (fewer registers per amplitude).
 template <typename T>
 static cudaError_t hpsi_tiled_t(const void* psi, void* lam, int n, int tb, bool realst, const HClass* classes,
                                 int nclasses, const HGroup* groups, const void* chunks, double* partials,
                                 unsigned* counter, double* out, int nblocks, cudaStream_t s) {
-  switch (tb) {
-    case 10: return hpsi_tiled_e<T, 4>(psi, lam, n, realst, classes, nclasses, groups, chunks, partials, counter, out, nblocks, s);
-    case 11: return hpsi_tiled_e<T, 8>(psi, lam, n, realst, classes, nclasses, groups, chunks, partials, counter, out, nblocks, s);
-    default: return cudaErrorInvalidValue;
-  }
+  const auto f = tb == 11 && realst ? hpsi_tiled_e<T, 8, true>
+                 : tb == 10         ? (realst ? hpsi_tiled_e<T, 4, true> : hpsi_tiled_e<T, 4, false>)
+                                    : nullptr;
+  if (!f) return cudaErrorInvalidValue;
+  return f(psi, lam, n, classes, nclasses, groups, chunks, partials, counter, out, nblocks, s);
 }
 cudaError_t launch_hpsi_tiled(const void* psi, void* lam, int n, qf_dtype dt, int tb, bool realst,
                               const HClass* classes, int nclasses, const HGroup* groups, const void* chunks,

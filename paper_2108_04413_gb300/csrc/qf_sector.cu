@@ -917,7 +917,7 @@ __global__ void __launch_bounds__(kRunThreads) k_run_itemmap(RunInfo run, const 
 // runs with a CTA barrier per block, 47 us here.
 constexpr int kPoolRuns = 40;  // runs described by one launch (kernel arguments stay under 4 KB)
 struct PoolRuns {
-  int n, slices;
+  int slices;
   RunInfo run[kPoolRuns];
 };
 template <typename T>
@@ -2156,9 +2156,9 @@ static cudaError_t overlaps_t(const void* psi, const RunInfo* runs, int nruns, c
   const size_t smem = (cm.cnt_o + (cnt_e + pr.slices - 1) / pr.slices) * sizeof(uint32_t);
   if (smem > (size_t)kMaxLists) return cudaErrorInvalidValue;
   for (int r0 = 0; r0 < nruns; r0 += kPoolRuns) {
-    pr.n = std::min(kPoolRuns, nruns - r0);
-    std::copy(runs + r0, runs + r0 + pr.n, pr.run);
-    const int nb = pr.run[pr.n - 1].b1 - pr.run[0].b0;
+    const int n = std::min(kPoolRuns, nruns - r0);
+    std::copy(runs + r0, runs + r0 + n, pr.run);
+    const int nb = pr.run[n - 1].b1 - pr.run[0].b0;
     k_pool_overlaps<T><<<nb * pr.slices, 256, smem, s>>>(static_cast<const V*>(psi), blks, partial, cm, pr);
     count_launch();
     const cudaError_t e = cudaGetLastError();
