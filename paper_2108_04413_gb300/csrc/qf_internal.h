@@ -97,8 +97,9 @@ struct TileArgs {
 // The indices off ^ (any sum of v[0..d-1]): where a state may be nonzero.  The v's have
 // distinct highest bits.  A determinant has d = 0, and a rotation adds its X mask to the
 // span, so a circuit's first rotations act on few amplitudes.
-// From 18 qubits on (below, a pass is bound by its launch): 28 qubits, 100 random rotations,
-// complex128: 111 ms visiting every tile, 84 ms; 27 qubits, 300, complex64: 36.6 and 33.8 ms.
+// From 18 qubits on (below, a pass is bound by its launch): 28 qubits, 100 random rotations in
+// list order, complex128: 111 ms visiting every tile, 84 ms the reached ones; 27 qubits, 300,
+// complex64: 36.6 and 33.8 ms (commuting rotations gathered as well: 76 to 82 and 32 ms).
 struct Support {
   int d;  // -1: unknown
   uint64_t off, v[QF_MAX_QUBITS];

@@ -778,9 +778,11 @@ __global__ void __launch_bounds__(256) k_pairs(typename Cx<T>::V* __restrict__ p
 // step's one-electron flips, each with a Z on every other qubit; its diagonal): on the pair
 // (b, b ^ x) their product is one rotation by phi(b), the sum of the angles with signs
 // (-1)^{popc(z & b)}, added as whole numbers (phase_turns): the sum of all less twice those
-// of odd parity.  Bound by the integer pipes, about ten operations a string, and one FP64
-// sine and cosine a pair, where a rotation each takes four multiply-adds a string and pair.
-// Trotter step at 20 qubits, 3631 strings in 91 runs: 7.8 ms as tile passes, 1.4 ms.
+// of odd parity: about ten integer operations a string and one FP64 sine and cosine a pair,
+// where a rotation each takes four FP64 multiply-adds a string and pair.  At 20 qubits a
+// launch takes 11 us, bound by its prologue and latency (barrier the top stall, FP64 pipe 18 %).
+// Trotter step at 20 qubits, 3631 strings in 91 runs: 7.8 ms as tile passes, 1.5 ms here, each
+// launch timed by itself; the whole step 5.91 ms with FP64 sums of the angles, 5.51 ms.
 __global__ void __launch_bounds__(256) k_phase_run(double2* __restrict__ psi, int n,
                                                    const __grid_constant__ PhaseArgs a) {
   __shared__ uint64_t turn[kPhaseMax];
@@ -1128,14 +1130,14 @@ __global__ void __launch_bounds__(256) k_expect_tiled(const typename Cx<T>::V* _
 
 // Passes (ExpPass): a CTA stages a tile of 2^S amplitudes (64 KB) in shared memory
 // with asynchronous copies and evaluates every group of the pass on it, so the
-// state is read once per pass instead of once per group (28 qubits, 500 strings: 53
-// reads instead of 440); three CTAs per SM overlap one's copies with the others'
+// state is read once per pass instead of once per group (28 qubits, 500 strings: 55
+// reads instead of 430); three CTAs per SM overlap one's copies with the others'
 // sums.
 // complex128 is bound by the FP64 pipe: two multiply-adds per pair and group, 75.6 ms
 // of the 91.5 ms that 25 qubits, 1500 terms take (236 ms in the per-group kernel).
 // complex64 is bound by shared-memory bandwidth (16 bytes per pair and group, 23 ms
 // of the 46 ms that 28 qubits, 500 terms take; 178 ms in the per-group kernel) and,
-// in passes of few groups, by the state's reads (53 reads: 17 ms); taking such passes
+// in passes of few groups, by the state's reads (55 reads: 18 ms); taking such passes
 // in turn with large ones tile by tile was slower (56 ms: spills).
 // complex64 sums stay in FP32 over four pairs, then join a float pair by TwoSum
 // (converted to FP64 once per tile).

@@ -429,8 +429,10 @@ __device__ void fill_binom_prefix(uint32_t (*Cs)[kBinom]) {
 // Programmatic dependent launch: a sweep launch may start while the previous
 // kernel of the stream finishes; it reads only plan data (descriptors, parts,
 // coefficients) before grid_dep_wait, which returns once that kernel has
-// completed and its writes are visible.  A kernel lets the next launch start
-// only after its own wait (so it never overlaps one two places before it).  Both
+// completed and its writes are visible.  A sweep lets the next launch start only
+// after its own wait; the block and run kernels of circuits do so before it,
+// which is as safe: every kernel launched with the attribute waits, for all of the
+// kernel before it and so for all before that, before it touches a state.  Both
 // are no-ops for a kernel launched without the attribute.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch_dependents() {
