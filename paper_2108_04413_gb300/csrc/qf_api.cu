@@ -80,7 +80,7 @@ struct ExpPlan {
   std::vector<qf_term> terms;        // the plan's terms (compared on every cache hit; tiled tables)
   std::vector<qf::ExpGroup> groups;  // host copies for the expectation passes
   std::vector<uint64_t> chunk_z;     // kChunkTerms masks per expectation chunk
-  double weight = 0.0;   // sum of |coeff|
+  double weight = -1.0;  // sum of |coeff| (on first use)
   bool has_odd = false;  // some term has an odd number of Y letters (imaginary phase)
   uint64_t last_use = 0; // the handle's call count at the plan's last use (least recently used goes first)
   // direct sector H|psi> tables (qf::SecDirect): 0 not tried yet, 1 built, -1 the
@@ -425,7 +425,16 @@ qf_status validate_masks(const qf_state* st, uint64_t x, uint64_t z) {
 // Pauli-sum plan: group by X mask, pack terms four per chunk with sign-pattern
 // tables (Eq. 18 evaluated pair by pair).
 
-qf_status get_plan(qf_state* st, const qf_term* terms, size_t nt, const ExpPlan** out) {
+std::vector<uint64_t> chunk_masks(const std::vector<qf::ExpChunk>& ech) {
+  std::vector<uint64_t> z;
+  z.reserve(ech.size() * qf::kChunkTerms);
+  for (const qf::ExpChunk& c : ech) z.insert(z.end(), c.z, c.z + qf::kChunkTerms);
+  return z;
+}
+
+// masks: a new plan keeps its chunks' masks on the host, for expectation passes (a plan made
+// without them reads them back when passes are first wanted).
+qf_status get_plan(qf_state* st, const qf_term* terms, size_t nt, const ExpPlan** out, bool masks = false) {
   auto same_terms = [&](const std::vector<qf_term>& seen) {
     return seen.size() == nt && (nt == 0 || std::memcmp(seen.data(), terms, nt * sizeof(qf_term)) == 0);
   };
@@ -733,9 +742,7 @@ qf_status get_plan(qf_state* st, const qf_term* terms, size_t nt, const ExpPlan*
     QF_CUDA(cudaStreamSynchronize(st->stream));
   }
   p.terms.assign(terms, terms + nt);
-  for (const qf_term& t : p.terms) p.weight += std::fabs(t.coeff);
-  p.chunk_z.reserve(ech.size() * qf::kChunkTerms);
-  for (const qf::ExpChunk& c : ech) p.chunk_z.insert(p.chunk_z.end(), c.z, c.z + qf::kChunkTerms);
+  if (masks) p.chunk_z = chunk_masks(ech);
   p.groups = std::move(groups);
   p.last_use = st->calls;
   auto res = st->plans.emplace(key, std::move(p));
@@ -862,6 +869,12 @@ void build_passes(const ExpPlan& p, int n, PassPlan* out) {
 qf_status ensure_passes(qf_state* st, ExpPlan* p, bool* use) {
   *use = p->npass >= 0;
   if (*use) return QF_OK;
+  if (p->chunk_z.empty()) {  // planned by a call that takes no passes
+    std::vector<qf::ExpChunk> ech(p->nchunks);
+    QF_CUDA(d2h(ech.data(), p->d_echunks, ech.size() * sizeof(qf::ExpChunk), st->stream));
+    QF_CUDA(cudaStreamSynchronize(st->stream));
+    p->chunk_z = chunk_masks(ech);
+  }
   PassPlan pp;
   if (st->dt == QF_C128)
     build_passes<double>(*p, st->n, &pp);
@@ -2564,14 +2577,14 @@ qf_status qf_expectation(qf_state* st, const qf_term* terms, size_t n_terms, dou
     return QF_OK;
   }
   trim_plans(st);
+  const bool general = st->sec_a < 0 && qf::launch_expect_passes && st->n >= kPassMinQubits;
   const ExpPlan* p = nullptr;
-  qf_status ps = get_plan(st, terms, n_terms, &p);
+  qf_status ps = get_plan(st, terms, n_terms, &p, general);
   if (ps != QF_OK) return ps;
   const int nb = qf::reduce_blocks(st->n, st->dt);
   int nsum = 1;  // device sums that make up the value
   bool passes = false;
-  if (st->sec_a < 0 && qf::launch_expect_passes && st->n >= kPassMinQubits &&
-      ((uint64_t)p->ngroups << st->n) >= kPassMinWork) {
+  if (general && ((uint64_t)p->ngroups << st->n) >= kPassMinWork) {
     qf_status xs = ensure_passes(st, const_cast<ExpPlan*>(p), &passes);
     if (xs != QF_OK) return xs;
   }
@@ -3105,6 +3118,11 @@ static qf_status energy_grad_impl(qf_state* st, uint64_t det, const qf_arot* ans
   // conj(lambda) psi, at most weight / scale^2 with a scale of 2^-31 or more, only for a
   // weight below 2^60 (and their rounding errors above 2^-60): past these, rotation by
   // rotation with FP64 products.
+  if (p && st->dt == QF_C64 && p->weight < 0.0) {
+    ExpPlan* pw = const_cast<ExpPlan*>(p);
+    pw->weight = 0.0;
+    for (const qf_term& t : p->terms) pw->weight += std::fabs(t.coeff);
+  }
   const bool tiles_back = n >= qf::kTileSmall && (st->dt == QF_C128 || !p || (p->weight < 0x1p60 && p->weight > 0x1p-60));
   // psi and lambda = H psi are both real when psi is real and H has no odd-Y term
   bool both_real = st->real && (!p || !p->has_odd);
