@@ -76,6 +76,7 @@ struct ExpPlan {
   void* d_pass = nullptr;
   size_t o_pgroup = 0, o_pchunk = 0, o_prest = 0;
   int npass = -1, nrest = 0;         // -1: not built yet
+  size_t pass_bytes = 0;             // their size, once planned (whether there is room is tried first)
   bool tiled = false;                // tiled H|psi> tables built (on first use)
   std::vector<qf_term> terms;        // the plan's terms (compared on every cache hit; tiled tables)
   std::vector<qf::ExpGroup> groups;  // host copies for the expectation passes
@@ -869,6 +870,13 @@ void build_passes(const ExpPlan& p, int n, PassPlan* out) {
 qf_status ensure_passes(qf_state* st, ExpPlan* p, bool* use) {
   *use = p->npass >= 0;
   if (*use) return QF_OK;
+  auto room = [&]() {
+    if (p->d_pass || cudaMalloc(&p->d_pass, p->pass_bytes) == cudaSuccess) return true;
+    cudaGetLastError();
+    p->d_pass = nullptr;
+    return false;
+  };
+  if (p->pass_bytes && !room()) return QF_OK;  // still none: the per-group kernel, without planning again
   if (p->chunk_z.empty()) {  // planned by a call that takes no passes
     std::vector<qf::ExpChunk> ech(p->nchunks);
     QF_CUDA(d2h(ech.data(), p->d_echunks, ech.size() * sizeof(qf::ExpChunk), st->stream));
@@ -886,13 +894,8 @@ qf_status ensure_passes(qf_state* st, ExpPlan* p, bool* use) {
   p->o_pgroup = up(b0);
   p->o_pchunk = p->o_pgroup + up(b1);
   p->o_prest = p->o_pchunk + up(b2);
-  cudaFree(p->d_pass);  // a failed upload's
-  p->d_pass = nullptr;
-  if (cudaMalloc(&p->d_pass, p->o_prest + up(b3)) != cudaSuccess) {
-    cudaGetLastError();
-    p->d_pass = nullptr;
-    return QF_OK;
-  }
+  p->pass_bytes = p->o_prest + up(b3);
+  if (!room()) return QF_OK;
   char* d = static_cast<char*>(p->d_pass);
   if (b0) QF_CUDA(h2d(d, pp.passes.data(), b0, st->stream));
   if (b1) QF_CUDA(h2d(d + p->o_pgroup, pp.groups.data(), b1, st->stream));
