@@ -118,7 +118,9 @@ qf_status qf_energy_grad(qf_state* st, uint64_t det, const qf_arot* ansatz, size
  * runs its first row through qf_energy_grad to do so), and when every block is
  * a real two-row sector block, H has direct sector tables and the sector's
  * psi and lambda fit in one CTA's shared memory (about 6000 members in
- * QF_C128, 12000 in QF_C64: up to 16 qubits at half filling), all rows run in
+ * QF_C128, 12000 in QF_C64: up to 16 qubits at half filling) and the device has
+ * room for the blocks' item map (4 bytes per member pair and block, at most 1 GB;
+ * kept with the handle, like the records of the rows), all rows run in
  * ONE kernel launch, one CTA per row, each holding its state in shared memory
  * through the forward blocks, H|psi> and the reverse blocks.  Otherwise the rows
  * run one after another through qf_energy_grad.  Errors as qf_energy_grad.
